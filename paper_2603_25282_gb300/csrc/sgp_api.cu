@@ -20,6 +20,7 @@
 #include "sgp_lab.cuh"
 #include "sgp_launch.cuh"
 #include "sgp_persist.cuh"
+#include "sgp_split.cuh"
 
 using namespace sgp;
 
@@ -332,6 +333,12 @@ struct sgp_ctx {
   const void* tmap_field[3] = {nullptr, nullptr, nullptr};   // the field a map was made for
   int* err_dev = nullptr;
   int var[3] = {0, 0, 0};                        // kernel variant per axis (x-pass, y, z lines)
+  // the kernel that variant 0 stands for on each axis (default_kernels), and
+  // whether the last work issued on the stream is a pass (which the next pass
+  // may follow as a dependent launch)
+  int def[3] = {0, 0, 0};
+  void* tws[3] = {nullptr, nullptr, nullptr};    // twiddles of their radix plan where it is not tw's
+  bool chain = false;
   double* t_dev = nullptr;
   double t = 0.0;
   std::vector<sgp_params> prm;      // per member
@@ -542,6 +549,7 @@ sgp_status get_tables(sgp_ctx* c, double delta, const LinTables** out) {
                                                     (long long)(nent * MT_STRIDE), (cplx<R>*)t.kz);
   }
   c->launches++;
+  c->chain = false;
   SGP_CUDA(c, cudaGetLastError());
   c->tables.push_back(t);
   *out = &c->tables.back();
@@ -617,6 +625,47 @@ bool plane_ok(const sgp_ctx* c) {
 // which has no plane pass.
 bool plane_pass(const sgp_ctx* c) { return c->var[0] == 5 && !c->rec; }
 
+// What variant 0 of an axis stands for, by the size of the whole batch (pts
+// grid points), the precision and the line length; measured per TS2 step on
+// the GB300 (plain variant 0 -> the choice, us):
+//   component-parallel passes for grids of few lines: FP32 2D up to 192 Ki
+//     points (64^2 22 -> 5, 256^2 32 -> 10, 384^2 44 -> 27; from 256 Ki points
+//     the others are ahead: 4 x 256^2 27 against 33), 3D below 128 Ki (48^3
+//     35 -> 28; 64 x 64 x 32 28 against 30); FP64, whose pipe the points keep
+//     busy in any kernel, for the x-pass wherever it exists (96 x 64 x 48 1002
+//     -> 856) and for 2D y-lines (192^2 395 -> 151; 3D z-lines 1002 -> 1113);
+//   FP32 2D otherwise: TMA tiles for the y-lines (768^2 104 -> 90 with x-pass
+//     geometry 1), geometry 1 for the x-pass except at 512 (16 x 256^2 75 ->
+//     72, 4 x 1024^2 367 -> 357, but 16 x 512^2 281 -> 288);
+//   FP32 3D otherwise: geometry 1 on every axis (128^3 230 -> 190).
+// With legacy (the groups of an ensemble, which stay comparable to the
+// persistent kernel bit for bit) variant 0 is the plain kernel.
+constexpr int kSplitPass = 100;
+PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder();
+
+void default_kernels(sgp_ctx* c, bool legacy) {
+  const long long pts = c->ntot * c->batch;
+  for (int a = 0; a < c->dim; ++a) {
+    c->def[a] = 0;
+    if (legacy) continue;
+    if (c->prec == SGP_F32) {
+      if (split_exists<float>(c->n[a]) && pts <= (c->dim == 2 ? 3LL << 16 : (1LL << 17) - 1))
+        c->def[a] = kSplitPass;
+      else if (c->dim == 3)
+        c->def[a] = 1;
+      else if (a == 0)
+        c->def[a] = c->n[0] == 512 ? 0 : 1;
+      else
+        c->def[a] = tensor_map_encoder() ? 4 : 1;
+    } else if (split_exists<double>(c->n[a]) && (a == 0 || c->dim == 2)) {
+      c->def[a] = kSplitPass;
+    }
+  }
+}
+
+// the kernel an axis runs: its variant, or what variant 0 stands for
+int axis_kernel(const sgp_ctx* c, int a) { return c->var[a] == 0 ? c->def[a] : c->var[a]; }
+
 template <typename R>
 XPassArgs<R> x_args(const sgp_ctx* c, void* field, int mode, double delta, double t_off) {
   XPassArgs<R> a{};
@@ -657,7 +706,13 @@ sgp_status x_pass_on(sgp_ctx* c, void* field, int mode, double delta, double t_o
   }
   c->launches++;
   ProfScope ps(c, PK_X);
-  SGP_CUDA(c, launch_xpass<R>(c->n[0], c->var[0], a, window_members(c), c->stream));
+  const bool dep = c->chain && !c->profiling;
+  c->chain = true;
+  if (axis_kernel(c, 0) == kSplitPass) {
+    if (c->tws[0]) a.tw = (const TwE<R>*)c->tws[0];
+    SGP_CUDA(c, launch_xsplit<R>(c->n[0], a, window_members(c), dep, c->stream));
+  } else
+    SGP_CUDA(c, launch_xpass<R>(c->n[0], axis_kernel(c, 0), a, window_members(c), dep, c->stream));
   return SGP_OK;
 }
 
@@ -671,6 +726,7 @@ sgp_status xy_pass_on(sgp_ctx* c, void* field, int mode, double delta, double t_
     const XPassArgs<R> a = x_args<R>(c, field, mode, delta, t_off);
     c->launches++;
     ProfScope ps(c, PK_X);
+    c->chain = false;
     SGP_CUDA(c, launch_xyplane(c->n[0], a, (const TwE<R>*)c->tw[1], c->err_dev, c->n[2],
                                 window_members(c), c->stream));
     return SGP_OK;
@@ -733,19 +789,27 @@ sgp_status line_pass_on(sgp_ctx* c, void* field, int axis, int mode, const LinTa
     return SGP_OK;
   }
   if constexpr (sizeof(R) == 4) {
-    if (c->var[axis] == 4) {
+    if (axis_kernel(c, axis) == 4) {
       // the batch the window's field belongs to (member coordinates mc0 + m)
       char* batch_base = (char*)field - (size_t)c->win0 * 5 * c->ntot * c->elem;
       SGP_TRY(ensure_tmap(c, axis, batch_base));
       c->launches++;
       ProfScope ps(c, axis == 1 ? PK_Y : PK_Z);
-      SGP_CUDA(c, launch_linepass_tma(c->n[axis], a, c->tmap[axis], planes, window_members(c), c->stream));
+      const bool dep = c->chain && !c->profiling;
+      c->chain = true;
+      SGP_CUDA(c, launch_linepass_tma(c->n[axis], a, c->tmap[axis], planes, window_members(c), dep, c->stream));
       return SGP_OK;
     }
   }
   c->launches++;
   ProfScope ps(c, axis == 1 ? PK_Y : PK_Z);
-  SGP_CUDA(c, launch_linepass<R>(c->n[axis], c->var[axis], a, planes, window_members(c), c->stream));
+  const bool dep = c->chain && !c->profiling;
+  c->chain = true;
+  if (axis_kernel(c, axis) == kSplitPass) {
+    if (c->tws[axis]) a.tw = (const TwE<R>*)c->tws[axis];
+    SGP_CUDA(c, launch_lsplit<R>(c->n[axis], a, planes, window_members(c), dep, c->stream));
+  } else
+    SGP_CUDA(c, launch_linepass<R>(c->n[axis], axis_kernel(c, axis), a, planes, window_members(c), dep, c->stream));
   return SGP_OK;
 }
 
@@ -840,6 +904,7 @@ template <typename R>
 sgp_status emit_steps(sgp_ctx* c, long long nsteps, double dt, int scheme) {
   const std::vector<SubRec> subs = merged_substeps(scheme, nsteps, dt);
   bool xspec = false;
+  c->chain = false;
   for (size_t j = 0; j < subs.size(); ++j) {
     if (subs[j].kind == 'N') {
       int mode = XP_NL | (xspec ? XP_INV : 0);
@@ -953,6 +1018,7 @@ sgp_status run_steps(sgp_ctx* c, long long nsteps, double dt, int scheme) {
 template <typename R>
 sgp_status substep(sgp_ctx* c, int kind, double delta) {
   c->launches++;
+  c->chain = false;
   k_set_time<<<1, 1, 0, c->stream>>>(c->t_dev, c->t);
   SGP_CUDA(c, cudaGetLastError());
   if (kind == SGP_SUB_NONLINEAR) {
@@ -1152,6 +1218,7 @@ sgp_status adjoint_nonlinear(sgp_ctx* c, const void* phi, double delta, double t
   a.prows = adjoint_prows<R>(c);
   c->launches++;
   ProfScope ps(c, PK_X);
+  c->chain = false;
   SGP_CUDA(c, launch_xadj<R>(c->n[0], a, c->batch, c->stream));
   return SGP_OK;
 }
@@ -1198,6 +1265,7 @@ sgp_status linear_hooked(sgp_ctx* c, void* f, double delta, const AdjHook<R>& h)
   c->launches++;
   {
     ProfScope ps(c, axis == 1 ? PK_Y : PK_Z);
+    c->chain = false;
     SGP_CUDA(c, launch_linepass_adj<R>(c->n[axis], a, h, planes, c->batch, c->stream));
   }
   if (c->dim == 3) SGP_TRY(line_pass_on<R>(c, f, 1, LP_INV, nullptr));
@@ -1239,6 +1307,7 @@ std::vector<SubRec> segment_substeps(int scheme, long long n, double dt) {
 template <typename R>
 sgp_status emit_recompute(sgp_ctx* c, const std::vector<SubRec>& subs, char* seg, char* spec) {
   const size_t sb = state_bytes(c);
+  c->chain = false;
   size_t nl = 0;
   bool xspec = false;
   for (size_t j = 0; j < subs.size(); ++j) {
@@ -1251,6 +1320,7 @@ sgp_status emit_recompute(sgp_ctx* c, const std::vector<SubRec>& subs, char* seg
       a.tap = (cplx<R>*)(seg + sb * (j + 1));
       c->launches++;
       ProfScope ps(c, PK_X);
+      c->chain = false;
       SGP_CUDA(c, launch_xpass_tap<R>(c->n[0], a, c->batch, c->stream));
     } else {
       if (!xspec) SGP_TRY(x_pass_on<R>(c, seg, XP_FWD, 0.0, 0.0));
@@ -1274,6 +1344,7 @@ template <typename R>
 sgp_status emit_adjoint(sgp_ctx* c, const std::vector<SubRec>& subs, const char* seg, const char* spec) {
   AdjRec& r = c->adj;
   const size_t sb = state_bytes(c);
+  c->chain = false;
   size_t nl = 0;
   for (const SubRec& q : subs) nl += q.kind == 'L';
   bool xspec = false;
@@ -2024,6 +2095,16 @@ sgp_status sgp_create_grid(int dim, const int* n, const double* L, int batch, in
                         : (a == 0 ? prepare_xpass<double>(c->n[a]) : prepare_linepass<double>(c->n[a]));
     if (e != cudaSuccess) return bail(SGP_ECUDA, "kernel attributes", e);
   }
+  default_kernels(c, false);
+  for (int a = 0; a < dim && e == cudaSuccess; ++a) {
+    const int v = c->def[a];
+    if (v == kSplitPass)
+      e = prec == SGP_F32 ? (a == 0 ? prepare_xsplit<float>(c->n[a]) : prepare_lsplit<float>(c->n[a]))
+                          : (a == 0 ? prepare_xsplit<double>(c->n[a]) : prepare_lsplit<double>(c->n[a]));
+    else if (v)
+      e = a == 0 ? prepare_xpass<float>(c->n[a], v) : prepare_linepass<float>(c->n[a], v);
+  }
+  if (e != cudaSuccess) return bail(SGP_ECUDA, "kernel attributes", e);
   const size_t fbytes = (size_t)batch * 5 * c->ntot * c->elem;
   if ((e = dev_alloc(c, &c->field, fbytes)) != cudaSuccess)
     return bail(SGP_ENOMEM, "field allocation", e);
@@ -2037,6 +2118,15 @@ sgp_status sgp_create_grid(int dim, const int* n, const double* L, int batch, in
       k_twiddles_f32<<<(c->n[a] + 255) / 256, 256, 0, c->stream>>>(c->n[a], E, (TwE<float>*)c->tw[a]);
     else
       k_twiddles_f64<<<(c->n[a] + 255) / 256, 256, 0, c->stream>>>(c->n[a], E, (TwE<double>*)c->tw[a]);
+    c->launches++;
+    const int es = prec == SGP_F32 ? split_elems_rt<float>(c->n[a]) : split_elems_rt<double>(c->n[a]);
+    if (c->def[a] != kSplitPass || es == E) continue;
+    if ((e = dev_alloc(c, &c->tws[a], (size_t)c->n[a] * 16)) != cudaSuccess)
+      return bail(SGP_ENOMEM, "twiddle allocation", e);
+    if (prec == SGP_F32)
+      k_twiddles_f32<<<(c->n[a] + 255) / 256, 256, 0, c->stream>>>(c->n[a], es, (TwE<float>*)c->tws[a]);
+    else
+      k_twiddles_f64<<<(c->n[a] + 255) / 256, 256, 0, c->stream>>>(c->n[a], es, (TwE<double>*)c->tws[a]);
     c->launches++;
   }
   if ((e = dev_alloc(c, (void**)&c->t_dev, sizeof(double))) != cudaSuccess)
@@ -2360,6 +2450,7 @@ sgp_status sgp_destroy(sgp_ctx* c) {
   dev_free(c, c->field);
   for (void* t : c->tw) dev_free(c, t);
   for (void* t : c->tw4) dev_free(c, t);
+  for (void* t : c->tws) dev_free(c, t);
   dev_free(c, c->t_dev);
   dev_free(c, c->err_dev);
   dev_free(c, c->mp_dev);
@@ -2795,6 +2886,7 @@ sgp_status sgp_ensemble_create(int dim, int count, const int* n, const double* L
       sgp_ensemble_destroy(e);
       return efail(nullptr, st, "group %zu: %s", g, msg.c_str());
     }
+    default_kernels(c, true);
     e->groups.push_back(c);
   }
   cudaEventCreateWithFlags(&e->fork, cudaEventDisableTiming);

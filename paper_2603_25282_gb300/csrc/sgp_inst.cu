@@ -68,15 +68,14 @@ static cudaError_t xpass_prepare_n() {
 }
 
 template <int N>
-static cudaError_t xpass_n(const XPassArgs<Real>& a, int members, cudaStream_t s) {
+static cudaError_t xpass_n(const XPassArgs<Real>& a, int members, bool dependent, cudaStream_t s) {
   constexpr int E = variant_elems<Real, N, V>();
   constexpr int G = variant_geom<N, V, SGP_PART>();
   typedef XCfg<Real, N, E, G> Cfg;
   cudaError_t e = xpass_prepare_n<N>();
   if (e != cudaSuccess) return e;
   dim3 grid((a.rows + Cfg::ROWS - 1) / Cfg::ROWS, members);
-  k_xpass<Real, N, E, G><<<grid, Cfg::THREADS, Cfg::SMEM, s>>>(a);
-  return cudaGetLastError();
+  return launch_pass(k_xpass<Real, N, E, G>, grid, Cfg::THREADS, Cfg::SMEM, dependent, s, a);
 }
 
 template <>
@@ -93,11 +92,11 @@ cudaError_t prepare_xpass_v<Real, V>(int N) {
 }
 
 template <>
-cudaError_t launch_xpass_v<Real, V>(int N, const XPassArgs<Real>& a, int members, cudaStream_t s) {
+cudaError_t launch_xpass_v<Real, V>(int N, const XPassArgs<Real>& a, int members, bool dependent, cudaStream_t s) {
   switch (N) {
 #define SGP_CASE(NN) \
   case NN:           \
-    return xpass_n<NN>(a, members, s);
+    return xpass_n<NN>(a, members, dependent, s);
     SGP_FOR_EACH_VN(SGP_CASE)
 #undef SGP_CASE
     default:
@@ -170,22 +169,21 @@ cudaError_t prepare_xpass_wide<Real>(int N) {
 }
 
 template <int N>
-static cudaError_t xpass_wide_n(const XPassArgs<Real>& a, int members, cudaStream_t s) {
+static cudaError_t xpass_wide_n(const XPassArgs<Real>& a, int members, bool dependent, cudaStream_t s) {
   constexpr int E = elems_per_thread<Real, N>();
   typedef XCfg<Real, N, E, 2> Cfg;
   cudaError_t e = xpass_wide_prepare_n<N>();
   if (e != cudaSuccess) return e;
   dim3 grid((a.rows + Cfg::ROWS - 1) / Cfg::ROWS, members);
-  k_xpass_wide<Real, N, E><<<grid, kXWideThreads, Cfg::SMEM, s>>>(a);
-  return cudaGetLastError();
+  return launch_pass(k_xpass_wide<Real, N, E>, grid, kXWideThreads, Cfg::SMEM, dependent, s, a);
 }
 
 template <>
-cudaError_t launch_xpass_wide<Real>(int N, const XPassArgs<Real>& a, int members, cudaStream_t s) {
+cudaError_t launch_xpass_wide<Real>(int N, const XPassArgs<Real>& a, int members, bool dependent, cudaStream_t s) {
   switch (N) {
 #define SGP_CASE(NN) \
   case NN:           \
-    return xpass_wide_n<NN>(a, members, s);
+    return xpass_wide_n<NN>(a, members, dependent, s);
     SGP_FOR_EACH_N(SGP_CASE)
 #undef SGP_CASE
     default:
@@ -254,7 +252,7 @@ static cudaError_t linepass_prepare_n() {
 
 template <int N>
 static cudaError_t linepass_n(const LPassArgs<Real>& a, int planes, int members,
-                              cudaStream_t s) {
+                              bool dependent, cudaStream_t s) {
   constexpr int E = variant_elems<Real, N, V>();
   constexpr int G = variant_geom<N, V, SGP_PART>();
   typedef LCfg<Real, N, E, G> Cfg;
@@ -263,8 +261,7 @@ static cudaError_t linepass_n(const LPassArgs<Real>& a, int planes, int members,
   dim3 grid((a.nx + Cfg::TILE - 1) / Cfg::TILE, planes, members);
   // the mode-table entries in shared memory when the pass mixes
   const size_t smem = Cfg::SMEM + line_table_bytes<Cfg>(a.mode, a.axis);
-  k_linepass<Real, N, E, G><<<grid, Cfg::THREADS, smem, s>>>(a);
-  return cudaGetLastError();
+  return launch_pass(k_linepass<Real, N, E, G>, grid, Cfg::THREADS, smem, dependent, s, a);
 }
 
 template <>
@@ -282,11 +279,11 @@ cudaError_t prepare_linepass_v<Real, V>(int N) {
 
 template <>
 cudaError_t launch_linepass_v<Real, V>(int N, const LPassArgs<Real>& a, int planes, int members,
-                                       cudaStream_t s) {
+                                       bool dependent, cudaStream_t s) {
   switch (N) {
 #define SGP_CASE(NN) \
   case NN:           \
-    return linepass_n<NN>(a, planes, members, s);
+    return linepass_n<NN>(a, planes, members, dependent, s);
     SGP_FOR_EACH_VN(SGP_CASE)
 #undef SGP_CASE
     default:
@@ -308,15 +305,14 @@ static cudaError_t linepass_tma_prepare_n() {
 
 template <int N>
 static cudaError_t linepass_tma_n(const LPassArgs<Real>& a, const CUtensorMap& map, int planes, int members,
-                                  cudaStream_t s) {
+                                  bool dependent, cudaStream_t s) {
   constexpr int E = elems_per_thread<Real, N>();
   typedef LCfg<Real, N, E, 1> Cfg;
   cudaError_t e = linepass_tma_prepare_n<N>();
   if (e != cudaSuccess) return e;
   dim3 grid((a.nx + Cfg::TILE - 1) / Cfg::TILE, planes, members);
   const size_t smem = Cfg::TSMEM + line_table_bytes<Cfg>(a.mode, a.axis);
-  k_linepass_tma<Real, N, E, 1><<<grid, Cfg::THREADS, smem, s>>>(a, map);
-  return cudaGetLastError();
+  return launch_pass(k_linepass_tma<Real, N, E, 1>, grid, Cfg::THREADS, smem, dependent, s, a, map);
 }
 
 PassGeom linepass_geom_tma(int N) { return linepass_geom_v<Real, 1>(N); }
@@ -334,11 +330,11 @@ cudaError_t prepare_linepass_tma(int N) {
 }
 
 cudaError_t launch_linepass_tma(int N, const LPassArgs<Real>& a, const CUtensorMap& map, int planes,
-                                int members, cudaStream_t s) {
+                                int members, bool dependent, cudaStream_t s) {
   switch (N) {
 #define SGP_CASE(NN) \
   case NN:           \
-    return linepass_tma_n<NN>(a, map, planes, members, s);
+    return linepass_tma_n<NN>(a, map, planes, members, dependent, s);
     SGP_FOR_EACH_N(SGP_CASE)
 #undef SGP_CASE
     default:

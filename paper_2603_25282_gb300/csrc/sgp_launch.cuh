@@ -34,6 +34,8 @@ inline bool supported_n(int n) {
 // chooses from):
 //   0  default geometry (x-pass: about 256 threads per CTA; line pass: up
 //      to 512 threads, TILE >= 4 FP32 / 2 FP64 columns) and radix plan
+//      (a context takes for it what suits its size: default_kernels in
+//      sgp_api.cu, with the component-parallel passes of sgp_split.cuh)
 //   1  CTAs of about half the threads (line pass: TILE down to 1)
 //   2  CTAs of about a quarter of the threads
 //   3  FP32 only.  N a power of two: radix-4 plan (4 elements per thread
@@ -82,19 +84,38 @@ struct PassGeom {
   size_t smem;
 };
 
+// Launch of a pass kernel; dependent: it may begin while the pass before it on
+// the stream is at work (the kernel waits in pdl_wait before it touches the
+// field).
+template <typename K, typename... A>
+inline cudaError_t launch_pass(K kern, dim3 grid, int threads, size_t smem, bool dependent, cudaStream_t s,
+                               const A&... a) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = dependent ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, a...);
+}
+
 // Per-variant entry points (explicitly instantiated in sgp_inst.cu).
 template <typename R, int V> PassGeom xpass_geom_v(int N);
 template <typename R, int V> PassGeom linepass_geom_v(int N);
 template <typename R, int V> cudaError_t prepare_xpass_v(int N);
 template <typename R, int V> cudaError_t prepare_linepass_v(int N);
 template <typename R, int V>
-cudaError_t launch_xpass_v(int N, const XPassArgs<R>& a, int members, cudaStream_t s);
+cudaError_t launch_xpass_v(int N, const XPassArgs<R>& a, int members, bool dependent, cudaStream_t s);
 template <typename R, int V>
 cudaError_t launch_linepass_v(int N, const LPassArgs<R>& a, int planes, int members,
-                              cudaStream_t s);
+                              bool dependent, cudaStream_t s);
 // Variant 4 of the line pass (tile loads by tensor copies over `map`).
 cudaError_t launch_linepass_tma(int N, const LPassArgs<float>& a, const CUtensorMap& map, int planes,
-                                int members, cudaStream_t s);
+                                int members, bool dependent, cudaStream_t s);
 cudaError_t prepare_linepass_tma(int N);
 PassGeom linepass_geom_tma(int N);
 // Variant 5 of the x-pass: the xy-plane pass over `planes` z planes of
@@ -105,7 +126,7 @@ cudaError_t launch_xyplane(int N, const XPassArgs<float>& a, const TwE<float>* t
 cudaError_t prepare_xyplane(int N);
 // Variant 6 of the x-pass (k_xpass_wide).
 template <typename R>
-cudaError_t launch_xpass_wide(int N, const XPassArgs<R>& a, int members, cudaStream_t s);
+cudaError_t launch_xpass_wide(int N, const XPassArgs<R>& a, int members, bool dependent, cudaStream_t s);
 template <typename R>
 cudaError_t prepare_xpass_wide(int N);
 
@@ -175,17 +196,17 @@ inline cudaError_t prepare_linepass(int N, int V = 0) {
 #undef SGP_C
 }
 template <typename R>
-inline cudaError_t launch_xpass(int N, int V, const XPassArgs<R>& a, int members, cudaStream_t s) {
-  if (V == 6) return launch_xpass_wide<R>(N, a, members, s);
-#define SGP_C(v) launch_xpass_v<R, v>(N, a, members, s)
+inline cudaError_t launch_xpass(int N, int V, const XPassArgs<R>& a, int members, bool dependent, cudaStream_t s) {
+  if (V == 6) return launch_xpass_wide<R>(N, a, members, dependent, s);
+#define SGP_C(v) launch_xpass_v<R, v>(N, a, members, dependent, s)
   SGP_VARIANT_SWITCH_X(V, SGP_C, cudaErrorInvalidValue)
 #undef SGP_C
 }
 // Variants 0-3 of the line pass (variant 4 goes through launch_linepass_tma).
 template <typename R>
 inline cudaError_t launch_linepass(int N, int V, const LPassArgs<R>& a, int planes, int members,
-                                   cudaStream_t s) {
-#define SGP_C(v) launch_linepass_v<R, v>(N, a, planes, members, s)
+                                   bool dependent, cudaStream_t s) {
+#define SGP_C(v) launch_linepass_v<R, v>(N, a, planes, members, dependent, s)
   SGP_VARIANT_SWITCH(V, SGP_C, cudaErrorInvalidValue)
 #undef SGP_C
 }
