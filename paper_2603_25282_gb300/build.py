@@ -27,8 +27,8 @@ UNITS = [
     ("api", "sgp_api.cu", []),
     ("adjoint_flo", "sgp_adjoint.cu", ["-DSGP_REAL=float", "-DSGP_REDUCE_PARAMS=1"]),
     ("adjoint_dou", "sgp_adjoint.cu", ["-DSGP_REAL=double"]),
-    ("split_flo", "sgp_split.cu", ["-DSGP_REAL=float"]),
-    ("split_dou", "sgp_split.cu", ["-DSGP_REAL=double"]),
+    ("split", "sgp_split.cu", []),
+    ("fix", "sgp_fix.cu", []),
     ("lab", "sgp_lab.cu", []),
     ("persist_flo", "sgp_persist.cu", ["-DSGP_REAL=float", "-DSGP_PERSIST_DEFINE_SUPPORTED=1"]),
     ("persist_dou", "sgp_persist.cu", ["-DSGP_REAL=double"]),

@@ -20,7 +20,7 @@
 #include "sgp_lab.cuh"
 #include "sgp_launch.cuh"
 #include "sgp_persist.cuh"
-#include "sgp_split.cuh"
+#include "sgp_fix.cuh"
 
 using namespace sgp;
 
@@ -631,16 +631,17 @@ bool plane_pass(const sgp_ctx* c) { return c->var[0] == 5 && !c->rec; }
 //   component-parallel passes for grids of few lines: FP32 2D up to 192 Ki
 //     points (64^2 22 -> 5, 256^2 32 -> 10, 384^2 44 -> 27; from 256 Ki points
 //     the others are ahead: 4 x 256^2 27 against 33), 3D below 128 Ki (48^3
-//     35 -> 28; 64 x 64 x 32 28 against 30); FP64, whose pipe the points keep
-//     busy in any kernel, for the x-pass wherever it exists (96 x 64 x 48 1002
-//     -> 856) and for 2D y-lines (192^2 395 -> 151; 3D z-lines 1002 -> 1113);
+//     35 -> 28; 64 x 64 x 32 28 against 30);
+//   FP64 everywhere (fixed-point transforms, sgp_fix.cuh: 64^2 229 -> 50, 8 x
+//     512^2 5300 -> 2500, 128^3 5510 -> 2610), with one line per CTA while that
+//     gives no more than four CTAs an SM;
 //   FP32 2D otherwise: TMA tiles for the y-lines (768^2 104 -> 90 with x-pass
 //     geometry 1), geometry 1 for the x-pass except at 512 (16 x 256^2 75 ->
 //     72, 4 x 1024^2 367 -> 357, but 16 x 512^2 281 -> 288);
 //   FP32 3D otherwise: geometry 1 on every axis (128^3 230 -> 190).
 // With legacy (the groups of an ensemble, which stay comparable to the
 // persistent kernel bit for bit) variant 0 is the plain kernel.
-constexpr int kSplitPass = 100;
+constexpr int kSplitPass = 100, kSplitMany = 101;
 PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder();
 
 void default_kernels(sgp_ctx* c, bool legacy) {
@@ -657,8 +658,8 @@ void default_kernels(sgp_ctx* c, bool legacy) {
         c->def[a] = c->n[0] == 512 ? 0 : 1;
       else
         c->def[a] = tensor_map_encoder() ? 4 : 1;
-    } else if (split_exists<double>(c->n[a]) && (a == 0 || c->dim == 2)) {
-      c->def[a] = kSplitPass;
+    } else if (split_exists<double>(c->n[a])) {
+      c->def[a] = pts / c->n[a] > 4 * 152 ? kSplitMany : kSplitPass;
     }
   }
 }
@@ -708,11 +709,12 @@ sgp_status x_pass_on(sgp_ctx* c, void* field, int mode, double delta, double t_o
   ProfScope ps(c, PK_X);
   const bool dep = c->chain && !c->profiling;
   c->chain = true;
-  if (axis_kernel(c, 0) == kSplitPass) {
+  const int kern = axis_kernel(c, 0);
+  if (kern >= kSplitPass) {
     if (c->tws[0]) a.tw = (const TwE<R>*)c->tws[0];
-    SGP_CUDA(c, launch_xsplit<R>(c->n[0], a, window_members(c), dep, c->stream));
+    SGP_CUDA(c, launch_xsplit<R>(c->n[0], kern != kSplitPass, a, window_members(c), dep, c->stream));
   } else
-    SGP_CUDA(c, launch_xpass<R>(c->n[0], axis_kernel(c, 0), a, window_members(c), dep, c->stream));
+    SGP_CUDA(c, launch_xpass<R>(c->n[0], kern, a, window_members(c), dep, c->stream));
   return SGP_OK;
 }
 
@@ -805,11 +807,12 @@ sgp_status line_pass_on(sgp_ctx* c, void* field, int axis, int mode, const LinTa
   ProfScope ps(c, axis == 1 ? PK_Y : PK_Z);
   const bool dep = c->chain && !c->profiling;
   c->chain = true;
-  if (axis_kernel(c, axis) == kSplitPass) {
+  const int kern = axis_kernel(c, axis);
+  if (kern >= kSplitPass) {
     if (c->tws[axis]) a.tw = (const TwE<R>*)c->tws[axis];
-    SGP_CUDA(c, launch_lsplit<R>(c->n[axis], a, planes, window_members(c), dep, c->stream));
+    SGP_CUDA(c, launch_lsplit<R>(c->n[axis], kern != kSplitPass, a, planes, window_members(c), dep, c->stream));
   } else
-    SGP_CUDA(c, launch_linepass<R>(c->n[axis], axis_kernel(c, axis), a, planes, window_members(c), dep, c->stream));
+    SGP_CUDA(c, launch_linepass<R>(c->n[axis], kern, a, planes, window_members(c), dep, c->stream));
   return SGP_OK;
 }
 
@@ -2098,9 +2101,10 @@ sgp_status sgp_create_grid(int dim, const int* n, const double* L, int batch, in
   default_kernels(c, false);
   for (int a = 0; a < dim && e == cudaSuccess; ++a) {
     const int v = c->def[a];
-    if (v == kSplitPass)
-      e = prec == SGP_F32 ? (a == 0 ? prepare_xsplit<float>(c->n[a]) : prepare_lsplit<float>(c->n[a]))
-                          : (a == 0 ? prepare_xsplit<double>(c->n[a]) : prepare_lsplit<double>(c->n[a]));
+    const bool many = v != kSplitPass;
+    if (v >= kSplitPass)
+      e = prec == SGP_F32 ? (a == 0 ? prepare_xsplit<float>(c->n[a], many) : prepare_lsplit<float>(c->n[a], many))
+                          : (a == 0 ? prepare_xsplit<double>(c->n[a], many) : prepare_lsplit<double>(c->n[a], many));
     else if (v)
       e = a == 0 ? prepare_xpass<float>(c->n[a], v) : prepare_linepass<float>(c->n[a], v);
   }
@@ -2119,14 +2123,14 @@ sgp_status sgp_create_grid(int dim, const int* n, const double* L, int batch, in
     else
       k_twiddles_f64<<<(c->n[a] + 255) / 256, 256, 0, c->stream>>>(c->n[a], E, (TwE<double>*)c->tw[a]);
     c->launches++;
-    const int es = prec == SGP_F32 ? split_elems_rt<float>(c->n[a]) : split_elems_rt<double>(c->n[a]);
-    if (c->def[a] != kSplitPass || es == E) continue;
+    if (c->def[a] < kSplitPass || (prec == SGP_F32 && split_elems_rt<float>(c->n[a]) == E)) continue;
     if ((e = dev_alloc(c, &c->tws[a], (size_t)c->n[a] * 16)) != cudaSuccess)
       return bail(SGP_ENOMEM, "twiddle allocation", e);
     if (prec == SGP_F32)
-      k_twiddles_f32<<<(c->n[a] + 255) / 256, 256, 0, c->stream>>>(c->n[a], es, (TwE<float>*)c->tws[a]);
-    else
-      k_twiddles_f64<<<(c->n[a] + 255) / 256, 256, 0, c->stream>>>(c->n[a], es, (TwE<double>*)c->tws[a]);
+      k_twiddles_f32<<<(c->n[a] + 255) / 256, 256, 0, c->stream>>>(c->n[a], split_elems_rt<float>(c->n[a]),
+                                                                  (TwE<float>*)c->tws[a]);
+    else if ((e = launch_fix_twiddles(c->n[a], (FixTw*)c->tws[a], c->stream)) != cudaSuccess)
+      return bail(SGP_ECUDA, "twiddles", e);
     c->launches++;
   }
   if ((e = dev_alloc(c, (void**)&c->t_dev, sizeof(double))) != cudaSuccess)

@@ -36,6 +36,7 @@ template <typename R> using cplx = typename cplx_t<R>::type;
 
 __device__ __forceinline__ float2 mkc(float a, float b) { return make_float2(a, b); }
 __device__ __forceinline__ double2 mkc(double a, double b) { return make_double2(a, b); }
+__device__ __forceinline__ longlong2 mkc(long long a, long long b) { return make_longlong2(a, b); }
 
 template <typename C> __device__ __forceinline__ C cadd(C a, C b) { return mkc(a.x + b.x, a.y + b.y); }
 template <typename C> __device__ __forceinline__ C csub(C a, C b) { return mkc(a.x - b.x, a.y - b.y); }
@@ -193,6 +194,33 @@ __device__ __forceinline__ float mul_rt3_half(float x) {
   return fmaf(x, 0.8660253882408142f, x * 1.5543625e-08f);
 }
 __device__ __forceinline__ double mul_rt3_half(double x) { return x * 0.86602540378443864676; }
+
+// The same on 64-bit integers (the fixed-point transforms of sgp_fix.cuh):
+// x as xh 2^32 + xl with xl signed
+__device__ __forceinline__ int fix_lo(long long x) { return (int)(unsigned)(unsigned long long)x; }
+__device__ __forceinline__ int fix_hi(long long x) {
+  return (int)(x >> 32) + (int)((unsigned)(unsigned long long)x >> 31);
+}
+__device__ __forceinline__ long long mad_wide(int a, int b, long long c) { return (long long)a * b + c; }
+
+// x k / 2^64 without the product of the low halves (below 1 unit); |x| < 2^62,
+// |k| < 2^63
+__device__ __forceinline__ long long fix_mulhi(long long x, int kh, int kl) {
+  const int xh = fix_hi(x), xl = fix_lo(x);
+  const long long t = mad_wide(xl, kh, (long long)xh * kl);
+  return mad_wide(xh, kh, t >> 32);
+}
+// sqrt(1/2) and sqrt(3)/2 in units of 2^-63, as hi 2^32 + lo (lo signed)
+constexpr long long kFixRtHalf = 6521908912666391106LL;
+constexpr long long kFixRt3Half = 7987674492471257551LL;
+__host__ __device__ constexpr int fix_chi(long long k) { return (int)((k + 0x80000000LL) >> 32); }
+__host__ __device__ constexpr int fix_clo(long long k) { return (int)(k - ((long long)fix_chi(k) << 32)); }
+__device__ __forceinline__ long long mul_rt_half(long long x) {
+  return fix_mulhi(x, fix_chi(kFixRtHalf), fix_clo(kFixRtHalf)) << 1;
+}
+__device__ __forceinline__ long long mul_rt3_half(long long x) {
+  return fix_mulhi(x, fix_chi(kFixRt3Half), fix_clo(kFixRt3Half)) << 1;
+}
 
 // Twiddle table entries.  FP32: W = hi + lo (both float2), applied with
 // tw_mul as one rounding of the product with the unevaluated sum, so the

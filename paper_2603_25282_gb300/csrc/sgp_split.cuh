@@ -44,8 +44,8 @@ struct SplitCfg {
   static constexpr int LP = line_pad_tile<R>(N, G);
   static constexpr int XCH = (LINES > 5 * G ? LINES : 5 * G) * LP;
   static constexpr size_t SMEM = sizeof(TwE<R>) * (size_t)N + sizeof(cplx<R>) * (size_t)XCH;
-  // registers: about 96 (FP32) or 128 (FP64) a thread
-  static constexpr int MINB0 = 65536 / (THREADS * (sizeof(R) == 4 ? 96 : 128));
+  // registers: about 96 a thread
+  static constexpr int MINB0 = 65536 / (THREADS * 96);
   static constexpr int MINB1 = (int)(220 * 1024 / SMEM);
   static constexpr int MINB = MINB0 < 1 ? 1 : (MINB0 < MINB1 ? MINB0 : (MINB1 < 1 ? 1 : MINB1));
 };
@@ -265,25 +265,24 @@ k_lsplit(LPassArgs<R> a) {
 template <typename R, int N>
 constexpr int split_rows() { return N % 32 == 0 ? 1 : 2; }
 template <typename R, int N>
-constexpr int split_cols() { return sizeof(R) == 4 && N <= 512 ? 2 : 1; }
+constexpr int split_cols() { return N <= 512 ? 2 : 1; }
 // Elements per thread: those of the other passes, except 12 for N = 3*2^k:
 // radix 6 then 4s (192 = 6*4*4*2) instead of 6 then 2s (192 = 6*2*2*2*2*2), so
 // two stages fewer or more; one component's 12 elements are few registers.
 template <typename R, int N>
-constexpr int split_elems() { return N % 3 == 0 ? 12 : sizeof(R) == 4 ? 8 : 4; }
-// FP64 lines of more elements fill the FP64 pipe without being split
-template <typename R, int N>
-constexpr bool split_has() { return sizeof(R) == 4 || N <= 384; }
-
-// Launchers (sgp_split.cu, one unit per precision).  dependent: the launch
-// may begin while the pass before it on the stream is at work.
+constexpr int split_elems() { return N % 3 == 0 ? 12 : 8; }
+// Launchers: FP32 here (sgp_split.cu); in FP64 the component-parallel passes
+// are those of sgp_fix.cuh (sgp_fix.cu).  dependent: the launch may begin
+// while the pass before it on the stream is at work.  many (FP64): enough
+// lines for CTAs of several.
 template <typename R> bool split_exists(int N);
 template <typename R> int split_elems_rt(int N);
-template <typename R> cudaError_t prepare_xsplit(int N);
-template <typename R> cudaError_t prepare_lsplit(int N);
+template <typename R> cudaError_t prepare_xsplit(int N, bool many);
+template <typename R> cudaError_t prepare_lsplit(int N, bool many);
 template <typename R>
-cudaError_t launch_xsplit(int N, const XPassArgs<R>& a, int members, bool dependent, cudaStream_t s);
+cudaError_t launch_xsplit(int N, bool many, const XPassArgs<R>& a, int members, bool dependent, cudaStream_t s);
 template <typename R>
-cudaError_t launch_lsplit(int N, const LPassArgs<R>& a, int planes, int members, bool dependent, cudaStream_t s);
+cudaError_t launch_lsplit(int N, bool many, const LPassArgs<R>& a, int planes, int members, bool dependent,
+                          cudaStream_t s);
 
 }  // namespace sgp

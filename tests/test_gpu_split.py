@@ -85,3 +85,76 @@ def test_host_windows_match():
         want = c.get_state()
         for chunks in (1, 2, 5):
             assert np.array_equal(c.step_host(host, 0.0, 3, 1e-3, "ts2", chunks=chunks), want)
+
+
+# ---------------------------------------------------------------------------
+# the fixed-point transforms of the FP64 passes
+# ---------------------------------------------------------------------------
+def linear(f, n, plan=None, delta=0.03):
+    with sgp.Context(n, 6.0, prec="f64") as c:
+        c.set_params(**PRM)
+        if plan:
+            c.set_plan(plan)
+        c.set_state(f[None].copy(), 0.0)
+        c.substep("linear", delta)
+        return c.get_state()[0]
+
+
+@pytest.mark.parametrize("n", [(64, 48), (96, 32), (512, 16), (16, 384)])
+def test_fixed_point_lines(n):
+    """Lines of very different content: unstructured, one element, one
+    component far below the others, zeros; and every power-of-two scale of a
+    field (the common exponent of a line) gives the scaled result bit for bit."""
+    f = inputs.random_field(n, 5)
+    one = np.zeros_like(f)
+    one[2, 3, 5] = 1.5 - 0.5j
+    low = f.copy()
+    low[3] *= 1e-18
+    for g in (f, one, low):
+        assert rel(linear(g, n), linear(g, n, plan=(1, 1))) < TOL["f64"]
+    assert not linear(np.zeros_like(f), n).any()
+    want = linear(f, n)
+    for k in (-900, -40, 300, 900):
+        assert np.array_equal(linear(f * 2.0 ** k, n), want * 2.0 ** k), k
+    # components that do not mix keep their own relative accuracy
+    with sgp.Context(n, 6.0, prec="f64") as c:
+        c.set_params(omega=0.0, gamma=0.0)
+        c.set_state(low[None].copy(), 0.0)
+        c.substep("linear", 0.03)
+        got = c.get_state()[0]
+        c.set_plan((1, 1))
+        c.set_state(low[None].copy(), 0.0)
+        c.substep("linear", 0.03)
+        assert rel(got[3], c.get_state()[0][3]) < TOL["f64"]
+
+
+def test_fixed_point_not_finite():
+    """A NaN or an infinity leaves nothing finite, as in the FP64 transforms,
+    and the next state is clean again."""
+    n = (48, 64)
+    f = inputs.random_field(n, 5)
+    for bad in (np.nan, np.inf, -np.inf):
+        g = f.copy()
+        g[1, 7, 9] = bad
+        assert not np.isfinite(linear(g, n)).any()
+        assert not np.isfinite(linear(g, n, plan=(1, 1))).any()
+    assert np.isfinite(linear(f, n)).all()
+
+
+def test_flow_tiers():
+    """FP64 flow at one substep on every branch of its angles: Taylor degrees 3
+    to 6 of the spin rotation and past them, both forms of the singlet and of
+    the phase, against the plain kernels."""
+    n = (32, 16)
+    f = inputs.random_field(n, 8, scale=0.3)
+    for c1 in (0.0, 1e-4, 1e-3, 5e-3, 1e-2, 2.0, 40.0):
+        for c0, c2 in ((1.0, 0.01), (100.0, 2.0), (900.0, -300.0)):
+            out = []
+            for plan in ((0, 0), (1, 1)):
+                with sgp.Context(n, 6.0, prec="f64") as c:
+                    c.set_params(omega=0.3, gamma=0.5, c0=c0, c1=c1, c2=c2, gx=1.0, gy=1.5)
+                    c.set_plan(plan)
+                    c.set_state(f[None].copy(), 0.4)
+                    c.substep("nonlinear", 0.01)
+                    out.append(c.get_state())
+            assert rel(out[0], out[1]) < TOL["f64"], (c0, c1, c2)
