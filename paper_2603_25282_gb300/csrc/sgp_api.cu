@@ -1187,13 +1187,28 @@ sgp_status record_steps(sgp_ctx* c, long long nsteps, double dt, int scheme, lon
 // Rows of the parameter partials per member: one per CTA of the adjoint
 // x-pass, then one per CTA of the line pass that holds the full transform
 // (y lines in 2D, z lines in 3D).
+// On grids whose passes are the FP32 component-parallel ones, a gradient's are too.
+bool adj_split(const sgp_ctx* c) {
+  if (c->prec != SGP_F32) return false;
+  for (int a = 0; a < c->dim; ++a)
+    if (c->def[a] != kSplitPass) return false;
+  return true;
+}
+template <typename R>
+int adjoint_xrows(const sgp_ctx* c) {
+  const int rows = c->n[1] * c->n[2];
+  return adj_split(c) ? xsplit_ctas(c->n[0], rows) : xadj_ctas<R>(c->n[0], rows);
+}
+template <typename R>
+int adjoint_tiles(const sgp_ctx* c) {
+  const int axis = c->dim == 2 ? 1 : 2;
+  return adj_split(c) ? lsplit_tiles(c->n[axis], c->n[0]) : linepass_adj_tiles<R>(c->n[axis], c->n[0]);
+}
 template <typename R>
 int adjoint_prows(const sgp_ctx* c) {
-  const int axis = c->dim == 2 ? 1 : 2;
   const int planes = c->dim == 2 ? c->n[2] : c->n[1];
-  return xadj_ctas<R>(c->n[0], c->n[1] * c->n[2]) + linepass_adj_tiles<R>(c->n[axis], c->n[0]) * planes;
+  return adjoint_xrows<R>(c) + adjoint_tiles<R>(c) * planes;
 }
-
 // g <- (D N_d(Phi_in))^T g at Phi_out = phi (physical space), plus the
 // parameter terms; with XP_INV g comes in x-spectral (the inverse
 // x-transform first), with XP_FWD it leaves x-spectral
@@ -1221,6 +1236,15 @@ sgp_status adjoint_nonlinear(sgp_ctx* c, const void* phi, double delta, double t
   a.prows = adjoint_prows<R>(c);
   c->launches++;
   ProfScope ps(c, PK_X);
+  if constexpr (sizeof(R) == 4) {
+    if (adj_split(c)) {
+      const bool dep = c->chain && !c->profiling;
+      c->chain = true;
+      if (c->tws[0]) a.tw = (const TwE<R>*)c->tws[0];
+      SGP_CUDA(c, launch_xadj_split(c->n[0], a, c->batch, dep, c->stream));
+      return SGP_OK;
+    }
+  }
   c->chain = false;
   SGP_CUDA(c, launch_xadj<R>(c->n[0], a, c->batch, c->stream));
   return SGP_OK;
@@ -1268,8 +1292,19 @@ sgp_status linear_hooked(sgp_ctx* c, void* f, double delta, const AdjHook<R>& h)
   c->launches++;
   {
     ProfScope ps(c, axis == 1 ? PK_Y : PK_Z);
-    c->chain = false;
-    SGP_CUDA(c, launch_linepass_adj<R>(c->n[axis], a, h, planes, c->batch, c->stream));
+    bool done = false;
+    if constexpr (sizeof(R) == 4) {
+      if (adj_split(c)) {
+        const bool dep = c->chain && !c->profiling;
+        c->chain = done = true;
+        if (c->tws[axis]) a.tw = (const TwE<R>*)c->tws[axis];
+        SGP_CUDA(c, launch_lsplit_adj(c->n[axis], a, h, planes, c->batch, dep, c->stream));
+      }
+    }
+    if (!done) {
+      c->chain = false;
+      SGP_CUDA(c, launch_linepass_adj<R>(c->n[axis], a, h, planes, c->batch, c->stream));
+    }
   }
   if (c->dim == 3) SGP_TRY(line_pass_on<R>(c, f, 1, LP_INV, nullptr));
   return SGP_OK;
@@ -1286,9 +1321,8 @@ sgp_status adjoint_linear(sgp_ctx* c, double delta, const void* phi_tap) {
   h.mp = c->mp_dev;
   h.partials = c->adj.part;
   h.prows = adjoint_prows<R>(c);
-  h.prow0 = xadj_ctas<R>(c->n[0], c->n[1] * c->n[2]);
-  const int axis = c->dim == 2 ? 1 : 2;
-  h.tiles = linepass_adj_tiles<R>(c->n[axis], c->n[0]);
+  h.prow0 = adjoint_xrows<R>(c);
+  h.tiles = adjoint_tiles<R>(c);
   h.Lx = c->L[0];
   h.Ly = c->L[1];
   h.delta = delta;
@@ -1323,8 +1357,19 @@ sgp_status emit_recompute(sgp_ctx* c, const std::vector<SubRec>& subs, char* seg
       a.tap = (cplx<R>*)(seg + sb * (j + 1));
       c->launches++;
       ProfScope ps(c, PK_X);
-      c->chain = false;
-      SGP_CUDA(c, launch_xpass_tap<R>(c->n[0], a, c->batch, c->stream));
+      bool done = false;
+      if constexpr (sizeof(R) == 4) {
+        if (adj_split(c)) {
+          const bool dep = c->chain && !c->profiling;
+          c->chain = done = true;
+          if (c->tws[0]) a.tw = (const TwE<R>*)c->tws[0];
+          SGP_CUDA(c, launch_xsplit_tap(c->n[0], a, c->batch, dep, c->stream));
+        }
+      }
+      if (!done) {
+        c->chain = false;
+        SGP_CUDA(c, launch_xpass_tap<R>(c->n[0], a, c->batch, c->stream));
+      }
     } else {
       if (!xspec) SGP_TRY(x_pass_on<R>(c, seg, XP_FWD, 0.0, 0.0));
       xspec = true;
@@ -1546,6 +1591,7 @@ sgp_status backward_sweep_pipelined(sgp_ctx* c, const std::vector<SubRec>& full,
 template <typename R>
 sgp_status backward_sweep(sgp_ctx* c) {
   AdjRec& r = c->adj;
+  if (adj_split(c)) SGP_CUDA(c, prepare_adj_split(c->n[0], c->n[c->dim - 1]));   // not inside a capture
   const size_t sb = state_bytes(c);
   const auto seq = scheme_seq(r.scheme);
   // a segment buffer: the start state (the recomputation's working state),

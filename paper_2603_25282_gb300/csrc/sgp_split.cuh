@@ -16,6 +16,7 @@
 // the same run is still at work (programmatic dependent launch); the field is
 // read and written only after it.
 #pragma once
+#include "sgp_adjoint.cuh"
 #include "sgp_kernels.cuh"
 
 namespace sgp {
@@ -87,7 +88,7 @@ k_xsplit(XPassArgs<R> a) {
   for (int k = tid; k < N; k += Cfg::THREADS) tw[k] = a.tw[k];
   if ((a.mode & XP_NL) && tid == 0) {
     const MemberPrm& P = a.mp[member];
-    const double t = *a.t_base + a.t_off;
+    const double t = a.t_base ? *a.t_base + a.t_off : a.t_off;
     double sn, cs;
     sincos(P.omega * t, &sn, &cs);
     s_prm[0] = (R)cs;
@@ -170,9 +171,13 @@ k_xsplit(XPassArgs<R> a) {
 // ----------------------------------------------------------------------------
 // line pass
 // ----------------------------------------------------------------------------
-template <typename R, int N, int E, int G>
+// ADJ: the line pass of a gradient, with the work of AdjHook at every mode: the
+// sweep adds the Omega and gamma terms before the mix (h.spec, fetched with the
+// table entry), the recomputation keeps a copy after it (h.tap).
+struct NoAdj {};
+template <typename R, int N, int E, int G, bool ADJ, class H>
 __global__ void __launch_bounds__(SplitCfg<R, N, E, G>::THREADS, SplitCfg<R, N, E, G>::MINB)
-k_lsplit(LPassArgs<R> a) {
+k_lsplit(LPassArgs<R> a, H h) {
   typedef cplx<R> C;
   typedef SplitCfg<R, N, E, G> Cfg;
   constexpr int T = Cfg::T;
@@ -212,10 +217,25 @@ k_lsplit(LPassArgs<R> a) {
     kz = a.axis == 2 ? a.kz[pos] : mkc((R)0, (R)0);
     return load_mode_shared(a.mt + (size_t)member * a.mt_member, ap * (a.NY / 2 + 1) + aq);
   };
+  // element offset of mode p of component 0
+  auto element = [&](int p) -> size_t {
+    const int pos = p / G;
+    return (size_t)member * 5 * a.ntot + (size_t)plane * a.plane_stride + (size_t)pos * a.line_stride +
+           blockIdx.x * G + (p - pos * G);
+  };
   ModeEntry<R> m0{};
   int ps0 = 0, qs0 = 0;
   C kz0 = mkc((R)0, (R)0);
   if (mix && tid < Cfg::PTS) m0 = entry(tid, ps0, qs0, kz0);
+  // the transform of Phi_out at the mode: not written by the pass before
+  C sv[5];
+  if constexpr (ADJ) {
+    if (h.spec && tid < Cfg::PTS && blockIdx.x * G + tid % G < a.nx) {
+#pragma unroll
+      for (int c = 0; c < 5; ++c) sv[c] = h.spec[element(tid) + (size_t)c * a.ntot];
+    }
+  }
+  double acc[LPA_NT] = {0.0, 0.0};
   C v[1][E];
   pdl_wait();
   if (lane) {
@@ -239,9 +259,27 @@ k_lsplit(LPassArgs<R> a) {
       constexpr int CS = G * Cfg::LP;
       C q[5] = {pp[0], pp[CS], pp[2 * CS], pp[3 * CS], pp[4 * CS]};
       const C kh = mkc(m0.khr, m0.khi);
+      if constexpr (ADJ) {
+        if (h.spec && blockIdx.x * G + cl < a.nx) {
+          if (p != tid) {
+#pragma unroll
+            for (int c = 0; c < 5; ++c) sv[c] = h.spec[element(p) + (size_t)c * a.ntot];
+          }
+          const MemberPrm& P = h.mp[member];
+          constexpr double kPi = 3.14159265358979323846;
+          lin_param_mode<R>(q, sv, ps0, qs0, (R)P.gamma, (R)P.omega, (R)h.delta, (R)(kPi / h.Lx), (R)(kPi / h.Ly),
+                            acc);
+        }
+      }
       mix_entry<R>(q, a, m0, ps0, qs0, a.axis == 2 ? kinetic_z(kh, kz0) : kh);
 #pragma unroll
       for (int c = 0; c < 5; ++c) pp[c * CS] = q[c];
+      if constexpr (ADJ) {
+        if (h.tap && blockIdx.x * G + cl < a.nx) {
+#pragma unroll
+          for (int c = 0; c < 5; ++c) h.tap[element(p) + (size_t)c * a.ntot] = q[c];
+        }
+      }
     }
     __syncthreads();                    // every mode is done
     if (lane) {
@@ -256,6 +294,125 @@ k_lsplit(LPassArgs<R> a) {
 #pragma unroll
       for (int e = 0; e < E; ++e) base[e * step] = v[0][e];
     }
+  }
+  if constexpr (ADJ) {
+    if (h.spec) {                       // the same for every thread of the launch
+      __shared__ double red[(Cfg::THREADS / 32) * LPA_NT];
+      __shared__ double out[LPA_NT];
+      block_sums<LPA_NT>(acc, out, red);
+      if (tid < LPA_NT) {
+        double* row = h.partials + ((size_t)member * h.prows + h.prow0 + (size_t)plane * h.tiles + blockIdx.x) * GP_N;
+        row[tid == 0 ? GP_OMEGA : GP_GAMMA] += out[tid] * h.scale;
+      }
+    }
+  }
+}
+
+// ----------------------------------------------------------------------------
+// x-pass of the adjoint sweep (k_xadj with the components split)
+// ----------------------------------------------------------------------------
+template <typename R, int N, int E, int G>
+__global__ void __launch_bounds__(SplitCfg<R, N, E, G>::THREADS, 65536 / (SplitCfg<R, N, E, G>::THREADS * 128))
+k_xadj_split(XAdjArgs<R> a) {
+  typedef cplx<R> C;
+  typedef SplitCfg<R, N, E, G> Cfg;
+  constexpr int T = Cfg::T;
+  constexpr int GT = T <= 32 ? 32 : T;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  TwE<R>* tw = reinterpret_cast<TwE<R>*>(smem_raw);
+  C* xb = reinterpret_cast<C*>(tw + N);
+  __shared__ double s_rot[3];
+  __shared__ double red[(Cfg::THREADS / 32) * NLA_NT];
+  __shared__ double out[NLA_NT];
+  const bool early = gridDim.x * gridDim.y <= kSplitEarly;
+  if (early) pdl_trigger();
+  const int tid = threadIdx.x;
+  const int member = blockIdx.y;
+  for (int k = tid; k < N; k += Cfg::THREADS) tw[k] = a.tw[k];
+  if (tid == 0) {
+    const double t = *a.t_base + a.t_off;
+    sincos(a.mp[member].omega * t, &s_rot[1], &s_rot[0]);
+    s_rot[2] = t;
+  }
+  const size_t mo = (size_t)member * 5 * a.ntot;
+  const int line = tid / T;
+  const int i = tid - line * T;
+  const int comp = line / G, g = line - comp * G;
+  const int row = blockIdx.x * G + g;
+  const bool lane = tid < Cfg::FTP;
+  const bool valid = line < 5 * G && row < a.rows;
+  C* base = a.g + mo + (size_t)(valid ? comp : 0) * a.ntot + (size_t)(valid ? row : 0) * N + i;
+  C* b = xb + line * Cfg::LP;
+  const int bid = 1 + line;
+  C v[1][E];
+  // Phi_out at the thread's first point: not written by the pass before
+  C psi[5];
+  if (tid < Cfg::PTS && blockIdx.x * G + tid / N < a.rows) {
+    const C* pr = a.phi + mo + (size_t)(blockIdx.x * G) * N + tid;
+#pragma unroll
+    for (int c = 0; c < 5; ++c) psi[c] = pr[(size_t)c * a.ntot];
+  }
+  pdl_wait();
+  if (lane) {
+#pragma unroll
+    for (int e = 0; e < E; ++e) v[0][e] = valid ? base[T * e] : mkc((R)0, (R)0);
+  }
+  __syncthreads();                      // twiddles, s_rot
+  if (lane) {
+    if (a.mode & XP_INV) split_fft<R, N, E, +1, GT>(v, i, tw, b, bid);
+    group_sync<GT>(bid);                // the exchanges' reads are done
+#pragma unroll
+    for (int e = 0; e < E; ++e) b[padx<R>(i + T * e)] = v[0][e];
+  }
+  __syncthreads();                      // the rows are staged
+  double acc[NLA_NT] = {0.0, 0.0, 0.0, 0.0};
+  {
+    const MemberPrm& P = a.mp[member];
+    NLAdjPrm<R> q;
+    q.d = (R)a.delta;
+    q.c0p = (R)(P.c0 + P.c2 / 5.0);
+    q.c1 = (R)P.c1;
+    q.c2 = (R)P.c2;
+    q.tdgg = (R)(s_rot[2] * 2.0 * (P.gx2h - P.gy2h));
+    const R co = (R)s_rot[0], si = (R)s_rot[1];
+    const R gx2h = (R)P.gx2h, gy2h = (R)P.gy2h, gz2h = (R)P.gz2h;
+#pragma unroll 1
+    for (int p = tid; p < Cfg::PTS; p += Cfg::THREADS) {
+      const int r = p / N, j = p - r * N;
+      const int rw = blockIdx.x * G + r;
+      if (rw >= a.rows) break;          // p only grows
+      const int iy = rw % a.ny, iz = rw / a.ny;
+      const R x = a.x0 + (R)j * a.hx, y = a.y0 + (R)iy * a.hy, z = a.z0 + (R)iz * a.hz;
+      const R xr = co * x + si * y, yr = co * y - si * x;
+      const R V = gx2h * xr * xr + gy2h * yr * yr + gz2h * z * z;
+      if (p != tid) {
+        const C* pr = a.phi + mo + (size_t)rw * N + j;
+#pragma unroll
+        for (int c = 0; c < 5; ++c) psi[c] = pr[(size_t)c * a.ntot];
+      }
+      constexpr int CS = G * Cfg::LP;
+      C* sp = xb + split_slot<R, Cfg>(r, j);
+      C gp[5] = {sp[0], sp[CS], sp[2 * CS], sp[3 * CS], sp[4 * CS]};
+      nl_adjoint_point<R>(psi, gp, V, xr * yr, q, acc);
+#pragma unroll
+      for (int c = 0; c < 5; ++c) sp[c * CS] = gp[c];
+    }
+  }
+  __syncthreads();                      // every point is done
+  if (lane) {
+#pragma unroll
+    for (int e = 0; e < E; ++e) v[0][e] = b[padx<R>(i + T * e)];
+    if (!early) pdl_trigger();
+    if (a.mode & XP_FWD) split_fft<R, N, E, -1, GT>(v, i, tw, b, bid);
+    if (valid) {
+#pragma unroll
+      for (int e = 0; e < E; ++e) base[T * e] = v[0][e];
+    }
+  }
+  block_sums<NLA_NT>(acc, out, red);
+  if (tid < NLA_NT) {
+    const int slot[NLA_NT] = {GP_OMEGA, GP_C0, GP_C1, GP_C2};
+    a.partials[((size_t)member * a.prows + blockIdx.x) * GP_N + slot[tid]] += out[tid];
   }
 }
 
@@ -284,5 +441,15 @@ cudaError_t launch_xsplit(int N, bool many, const XPassArgs<R>& a, int members, 
 template <typename R>
 cudaError_t launch_lsplit(int N, bool many, const LPassArgs<R>& a, int planes, int members, bool dependent,
                           cudaStream_t s);
+// The passes of a gradient (FP32): the x-pass that copies its rows after the
+// flow to a.tap, the adjoint x-pass, the line pass with its hooks; CTAs per
+// member of the x-passes and columns' tiles per plane (rows of the partials).
+cudaError_t prepare_adj_split(int NX, int NL);
+cudaError_t launch_xsplit_tap(int N, const XPassArgs<float>& a, int members, bool dependent, cudaStream_t s);
+cudaError_t launch_xadj_split(int N, const XAdjArgs<float>& a, int members, bool dependent, cudaStream_t s);
+cudaError_t launch_lsplit_adj(int N, const LPassArgs<float>& a, const AdjHook<float>& h, int planes, int members,
+                              bool dependent, cudaStream_t s);
+int xsplit_ctas(int N, int rows);
+int lsplit_tiles(int N, int nx);
 
 }  // namespace sgp
