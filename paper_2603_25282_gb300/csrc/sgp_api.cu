@@ -337,6 +337,9 @@ struct sgp_ctx {
   // whether the last work issued on the stream is a pass (which the next pass
   // may follow as a dependent launch)
   int def[3] = {0, 0, 0};
+  // passes issued one by one carry the time themselves: the start of their run
+  bool own_time = false;
+  double run_t0 = 0.0;
   void* tws[3] = {nullptr, nullptr, nullptr};    // twiddles of their radix plan where it is not tw's
   bool chain = false;
   double* t_dev = nullptr;
@@ -684,8 +687,8 @@ XPassArgs<R> x_args(const sgp_ctx* c, void* field, int mode, double delta, doubl
   a.hz = c->dim == 3 ? (R)c->h[2] : (R)0;
   a.delta = (R)delta;
   a.mp = c->mp_dev + c->win0;
-  a.t_base = c->t_dev;
-  a.t_off = t_off;
+  a.t_base = c->own_time ? nullptr : c->t_dev;
+  a.t_off = c->own_time ? c->run_t0 + t_off : t_off;
   return a;
 }
 
@@ -896,7 +899,7 @@ std::vector<SubRec> merged_substeps(int scheme, long long n, double dt) {
 }
 
 // Issue nsteps of the composition from the device time *t_dev and advance
-// it by nsteps*dt, physical space in and out.  The merged substeps become
+// it by nsteps*dt (or, with own_time, from run_t0), physical space in and out.  The merged substeps become
 // passes: a nonlinear flow is an x-pass (inverse x-FFT if the field is
 // x-spectral, the flow, forward x-FFT if a linear flow follows); a linear
 // flow is the line passes on the x-spectral field (a forward x-pass first if
@@ -921,7 +924,7 @@ sgp_status emit_steps(sgp_ctx* c, long long nsteps, double dt, int scheme) {
     }
   }
   if (xspec) SGP_TRY(x_pass<R>(c, XP_INV, 0.0, 0.0));
-  if (c->rec) return SGP_OK;           // recording passes only; the caller advances the time
+  if (c->rec || c->own_time) return SGP_OK;   // the caller advances the time
   c->launches++;
   {
     ProfScope ps(c, PK_OTHER);
@@ -996,34 +999,47 @@ long long chunk_launches(const sgp_ctx* c, long long steps, int scheme) {
   return n + (xspec ? 1 : 0);
 }
 
+// Captured chunks keep the time on the device; the steps issued one by one,
+// here and in substep, carry it in their arguments, two launches fewer a run.
+struct OwnTime {
+  sgp_ctx* c;
+  OwnTime(sgp_ctx* ctx, double t0) : c(ctx) {
+    c->own_time = true;
+    c->run_t0 = t0;
+  }
+  ~OwnTime() { c->own_time = false; }
+};
+
 template <typename R>
 sgp_status run_steps(sgp_ctx* c, long long nsteps, double dt, int scheme) {
-  c->launches++;
-  {
-    ProfScope ps(c, PK_OTHER);
-    k_set_time<<<1, 1, 0, c->stream>>>(c->t_dev, c->t);
-  }
-  SGP_CUDA(c, cudaGetLastError());
   long long done = 0;
+  double t = c->t;
   if (c->use_graphs && !c->profiling && c->wcnt == 0 && nsteps >= 2 * kGraphChunk) {
+    c->launches++;
+    k_set_time<<<1, 1, 0, c->stream>>>(c->t_dev, c->t);
+    SGP_CUDA(c, cudaGetLastError());
     cudaGraphExec_t exec = nullptr;
     SGP_TRY(get_graph<R>(c, kGraphChunk, dt, scheme, &exec));
     const long long reps = nsteps / kGraphChunk;
-    for (long long r = 0; r < reps; ++r) SGP_CUDA(c, cudaGraphLaunch(exec, c->stream));
+    for (long long r = 0; r < reps; ++r) {
+      SGP_CUDA(c, cudaGraphLaunch(exec, c->stream));
+      t += (double)kGraphChunk * dt;          // as the chunk's k_add_time
+    }
     c->launches += reps * chunk_launches(c, kGraphChunk, scheme);
     done = reps * kGraphChunk;
   }
-  if (done < nsteps) SGP_TRY(emit_steps<R>(c, nsteps - done, dt, scheme));
+  if (done < nsteps) {
+    OwnTime own(c, t);
+    SGP_TRY(emit_steps<R>(c, nsteps - done, dt, scheme));
+  }
   c->t += (double)nsteps * dt;
   return SGP_OK;
 }
 
 template <typename R>
 sgp_status substep(sgp_ctx* c, int kind, double delta) {
-  c->launches++;
   c->chain = false;
-  k_set_time<<<1, 1, 0, c->stream>>>(c->t_dev, c->t);
-  SGP_CUDA(c, cudaGetLastError());
+  OwnTime own(c, c->t);
   if (kind == SGP_SUB_NONLINEAR) {
     SGP_TRY(x_pass<R>(c, XP_NL, delta, 0.0));
   } else {

@@ -512,7 +512,7 @@ __global__ void __launch_bounds__(FixCfg<N, G>::THREADS, FixCfg<N, G>::MINB) k_x
   for (int k = tid; k < N; k += Cfg::THREADS) tw[k] = reinterpret_cast<const FixTw*>(a.tw)[k];
   if ((a.mode & XP_NL) && tid == 0) {
     const MemberPrm& P = a.mp[member];
-    const double t = *a.t_base + a.t_off;
+    const double t = a.t_base ? *a.t_base + a.t_off : a.t_off;
     sincos(P.omega * t, &s_prm[1], &s_prm[0]);
     s_prm[2] = a.delta * (P.c0 + P.c2 / 5.0);
     s_prm[3] = a.delta * P.c1;

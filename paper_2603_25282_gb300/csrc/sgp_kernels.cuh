@@ -48,7 +48,8 @@ struct XPassArgs {
   int ny;
   int mode;
   R x0, hx, y0, hy, z0, hz;      // coordinates x_j = x0 + j*hx
-  // nonlinear flow over delta at time t = *t_base + t_off
+  // nonlinear flow over delta at time t = *t_base + t_off (t_off alone when
+  // t_base is null)
   R delta;
   const MemberPrm* mp;           // [batch]
   const double* t_base;
@@ -530,7 +531,7 @@ __device__ __forceinline__ void xpass_body(const XPassArgs<R>& a, int bx, int me
   for (int k = threadIdx.x; k < N; k += Cfg::THREADS) tw[k] = a.tw[k];
   if ((a.mode & XP_NL) && threadIdx.x == 0) {
     const MemberPrm& P = a.mp[member];
-    const double t = *a.t_base + a.t_off;
+    const double t = a.t_base ? *a.t_base + a.t_off : a.t_off;
     double sn, cs;
     sincos(P.omega * t, &sn, &cs);
     s_prm[0] = (R)cs;
@@ -622,7 +623,7 @@ __global__ void __launch_bounds__(kXWideThreads, 2) k_xpass_wide(XPassArgs<R> a)
   for (int k = tid; k < N; k += kXWideThreads) tw[k] = a.tw[k];
   if ((a.mode & XP_NL) && tid == 0) {
     const MemberPrm& P = a.mp[member];
-    const double t = *a.t_base + a.t_off;
+    const double t = a.t_base ? *a.t_base + a.t_off : a.t_off;
     double sn, cs;
     sincos(P.omega * t, &sn, &cs);
     s_prm[0] = (R)cs;
@@ -1012,7 +1013,7 @@ k_xyplane(XPassArgs<R> a, const TwE<R>* __restrict__ twy_g, int* err) {
   }
   if ((a.mode & XP_NL) && threadIdx.x == 0) {
     const MemberPrm& P = a.mp[member];
-    const double t = *a.t_base + a.t_off;
+    const double t = a.t_base ? *a.t_base + a.t_off : a.t_off;
     double sn, cs;
     sincos(P.omega * t, &sn, &cs);
     s_prm[0] = (R)cs;
