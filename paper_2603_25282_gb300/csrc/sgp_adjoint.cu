@@ -276,21 +276,8 @@ int linepass_adj_tiles<Real>(int N, int nx) {
 }
 
 #if SGP_REDUCE_PARAMS
-namespace {
-__global__ void k_reduce_params(const double* part, int nrows, int members, double* dp) {
-  const int id = blockIdx.x * blockDim.x + threadIdx.x;
-  if (id >= members * GP_N) return;
-  const int m = id / GP_N, k = id - m * GP_N;
-  const double* p = part + (size_t)m * nrows * GP_N + k;
-  double s = 0.0;
-  for (int b = 0; b < nrows; ++b) s += p[(size_t)b * GP_N];
-  dp[id] = s;
-}
-}  // namespace
-
 cudaError_t launch_reduce_params(const double* part, int nrows, int members, double* dp, cudaStream_t s) {
-  const int n = members * GP_N;
-  k_reduce_params<<<(n + 127) / 128, 128, 0, s>>>(part, nrows, members, dp);
+  k_reduce_partials<<<dim3(GP_N, members), kReduceThreads, 0, s>>>(part, nrows, GP_N, dp, GP_N, 0);
   return cudaGetLastError();
 }
 #endif

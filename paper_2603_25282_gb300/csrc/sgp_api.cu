@@ -1773,8 +1773,7 @@ sgp_status member_mass(sgp_ctx* c, std::vector<double>& out) {
   c->launches += 2;
   k_mass<R><<<dim3(kMassBlocks, c->batch), 256, 0, c->stream>>>((const cplx<R>*)c->field,
                                                                  5 * c->ntot, part);
-  k_reduce_partials<<<(c->batch + 127) / 128, 128, 0, c->stream>>>(part, kMassBlocks, 1, c->batch,
-                                                                   c->mass_dev, 1, 0);
+  k_reduce_partials<<<dim3(1, c->batch), kReduceThreads, 0, c->stream>>>(part, kMassBlocks, 1, c->mass_dev, 1, 0);
   SGP_CUDA(c, cudaGetLastError());
   out.resize(c->batch);
   SGP_CUDA(c, cudaMemcpyAsync(out.data(), c->mass_dev, sizeof(double) * c->batch,
@@ -2005,8 +2004,8 @@ sgp_status observables(sgp_ctx* c, sgp_obs* out) {
     SGP_CUDA(c, launch_obs_x<R>(NX, ax, c->batch, c->stream));
   }
   c->launches++;
-  k_reduce_partials<<<(c->batch * OBX_NT + 127) / 128, 128, 0, c->stream>>>(
-      c->partials, nbx, OBX_NT, c->batch, c->obs_dev, OB_NT, 0);
+  k_reduce_partials<<<dim3(OBX_NT, c->batch), kReduceThreads, 0, c->stream>>>(c->partials, nbx, OBX_NT, c->obs_dev,
+                                                                             OB_NT, 0);
   SGP_CUDA(c, cudaGetLastError());
   for (int axis = 1; axis < c->dim; ++axis) {
     const int NL = c->n[axis];
@@ -2038,9 +2037,8 @@ sgp_status observables(sgp_ctx* c, sgp_obs* out) {
       SGP_CUDA(c, launch_obs_line<R>(NL, al, planes, c->batch, c->stream));
     }
     c->launches++;
-    k_reduce_partials<<<(c->batch * OBL_NT + 127) / 128, 128, 0, c->stream>>>(
-        c->partials, al.nblocks, OBL_NT, c->batch, c->obs_dev, OB_NT,
-        axis == 1 ? OB_KY : OB_KZ);
+    k_reduce_partials<<<dim3(OBL_NT, c->batch), kReduceThreads, 0, c->stream>>>(
+        c->partials, al.nblocks, OBL_NT, c->obs_dev, OB_NT, axis == 1 ? OB_KY : OB_KZ);
     SGP_CUDA(c, cudaGetLastError());
   }
   std::vector<double> h((size_t)c->batch * OB_NT, 0.0);
@@ -3406,8 +3404,8 @@ sgp_status observables_static_impl(int dim, const int* nn, const double* LL, int
   ax.NX = n[0];
   if ((e = launch_obs_x<R>(n[0], ax, batch, stream)) != cudaSuccess)
     return static_fail(SGP_ECUDA, "obs_x: %s", cudaGetErrorString(e));
-  k_reduce_partials<<<(batch * OBX_NT + 127) / 128, 128, 0, stream>>>(
-      sc->partials, nbx, OBX_NT, batch, sc->sums, OB_NT, 0);
+  k_reduce_partials<<<dim3(OBX_NT, batch), kReduceThreads, 0, stream>>>(sc->partials, nbx, OBX_NT, sc->sums, OB_NT,
+                                                                       0);
   for (int axis = 1; axis < dim; ++axis) {
     const int NL = n[axis];
     const PassGeom gl = linepass_geom<R>(NL);
@@ -3433,8 +3431,8 @@ sgp_status observables_static_impl(int dim, const int* nn, const double* LL, int
     al.nblocks = ((n[0] + gl.rows_or_tile - 1) / gl.rows_or_tile) * planes;
     if ((e = launch_obs_line<R>(NL, al, planes, batch, stream)) != cudaSuccess)
       return static_fail(SGP_ECUDA, "obs_line: %s", cudaGetErrorString(e));
-    k_reduce_partials<<<(batch * OBL_NT + 127) / 128, 128, 0, stream>>>(
-        sc->partials, al.nblocks, OBL_NT, batch, sc->sums, OB_NT, axis == 1 ? OB_KY : OB_KZ);
+    k_reduce_partials<<<dim3(OBL_NT, batch), kReduceThreads, 0, stream>>>(
+        sc->partials, al.nblocks, OBL_NT, sc->sums, OB_NT, axis == 1 ? OB_KY : OB_KZ);
   }
   if ((e = cudaGetLastError()) != cudaSuccess)
     return static_fail(SGP_ECUDA, "launch: %s", cudaGetErrorString(e));
