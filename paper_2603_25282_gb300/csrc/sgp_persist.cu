@@ -108,8 +108,8 @@ k_ens_persistent(const PersistPass<R>* __restrict__ prog, const __grid_constant_
         const int tiles = line ? lay.lt[g] : lay.xt[g];
         const int rl = r - off[g];
         ml = rl / items;
-        tile0 = (rl - ml * items) * kTilesPerItem;
-        tile1 = tile0 + kTilesPerItem < tiles ? tile0 + kTilesPerItem : tiles;
+        tile0 = (rl - ml * items) * lay.tpi;
+        tile1 = tile0 + lay.tpi < tiles ? tile0 + lay.tpi : tiles;
         ent = p * lay.groups + g;
         slot = lay.base[g] + ml;
         const int need = ((p + 1) / 2) * lay.xi[g] + (p / 2) * lay.li[g];

@@ -34,12 +34,12 @@ struct PersistPass {
 // Shape of a program (kernel parameter): passes alternate x-pass, line
 // pass, x-pass, ... (2D), every x-pass has IX work items and every line
 // pass IL; inside a pass the groups' items follow each other.  A work item
-// is up to kTilesPerItem consecutive tiles of one member.
+// is up to tpi consecutive tiles of one member.
 constexpr int kPersistMaxGroups = 32;
-constexpr int kTilesPerItem = 2;
 struct PersistLayout {
   int IX, IL;                            // work items of an x-pass and of a line pass
   int groups;
+  int tpi;                               // tiles per work item
   int xoff[kPersistMaxGroups + 1];       // items of the groups before g in an x-pass
   int loff[kPersistMaxGroups + 1];       // the same in a line pass
   int xt[kPersistMaxGroups];             // tiles per member of an x-pass
