@@ -318,6 +318,7 @@ struct AdjHook {
   double* partials;
   int prows, prow0, tiles;
   double Lx, Ly, delta, scale;
+  __device__ __forceinline__ int groups() const { return spec ? 1 : 0; }
   // bytes of shared memory the hook stages: the tile of spec
   template <typename RR, int N, int TILE>
   static constexpr size_t smem_bytes() { return (size_t)5 * N * TILE * sizeof(cplx<RR>); }

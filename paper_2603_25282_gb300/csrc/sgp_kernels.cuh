@@ -456,6 +456,40 @@ struct XCfg {
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 
+// 16-byte asynchronous copy global -> shared (completes at cp_async_wait)
+__device__ __forceinline__ void cp_async16(void* dst_shared, const void* src_global) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst_shared);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src_global) : "memory");
+}
+// 8-byte asynchronous copy global -> shared (through L1)
+__device__ __forceinline__ void cp_async8(void* dst_shared, const void* src_global) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst_shared);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(src_global) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() {
+  asm volatile("cp.async.commit_group;\n" ::: "memory");
+}
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_all;\n" ::: "memory");
+}
+// the groups committed before the last n are complete
+template <int n>
+__device__ __forceinline__ void cp_async_wait_group() {
+  asm volatile("cp.async.wait_group %0;\n" ::"n"(n) : "memory");
+}
+
+// The twiddle table to shared memory: asynchronous copies (one group), plain
+// loads in the persistent kernel (there the copies measured 1% slower).
+template <bool CG, int THREADS, typename W>
+__device__ __forceinline__ void load_twiddles(W* dst, const W* src, int n) {
+  static_assert(sizeof(W) == 16, "16-byte pieces");
+  for (int k = threadIdx.x; k < n; k += THREADS) {
+    if constexpr (CG) dst[k] = src[k];
+    else cp_async16(dst + k, src + k);
+  }
+  if constexpr (!CG) cp_async_commit();
+}
+
 // x-pass: rows of all five components.  The nonlinear flow runs on the rows
 // staged in shared memory between the two transforms, as a plain loop over
 // points: one copy of its code (the unrolled form did not fit the
@@ -528,36 +562,50 @@ __device__ __forceinline__ void xpass_body(const XPassArgs<R>& a, int bx, int me
   __shared__ R s_yz[Cfg::ROWS][2];    // y and z of the CTA's rows
   const int g = threadIdx.x / T;
   const int i = threadIdx.x - g * T;
-  for (int k = threadIdx.x; k < N; k += Cfg::THREADS) tw[k] = a.tw[k];
-  if ((a.mode & XP_NL) && threadIdx.x == 0) {
-    const MemberPrm& P = a.mp[member];
-    const double t = a.t_base ? *a.t_base + a.t_off : a.t_off;
-    double sn, cs;
-    sincos(P.omega * t, &sn, &cs);
-    s_prm[0] = (R)cs;
-    s_prm[1] = (R)sn;
-    s_prm[2] = (R)(P.c0 + P.c2 / 5.0);
-    s_prm[3] = (R)P.c1;
-    s_prm[4] = (R)P.c2;
-    s_prm[5] = (R)P.gx2h;
-    s_prm[6] = (R)P.gy2h;
-    s_prm[7] = (R)P.gz2h;
-  }
-  if ((a.mode & XP_NL) && threadIdx.x < Cfg::ROWS) {
-    const int rr = bx * Cfg::ROWS + threadIdx.x;
-    s_yz[threadIdx.x][0] = a.y0 + (R)(rr % a.ny) * a.hy;
-    s_yz[threadIdx.x][1] = a.z0 + (R)(rr / a.ny) * a.hz;
-  }
+  // the twiddles by asynchronous copies: loads whose values go to shared
+  // memory would hold the field loads back by an L2 round trip
+  load_twiddles<CG, Cfg::THREADS>(tw, a.tw, N);
+  auto constants = [&]() {
+    if ((a.mode & XP_NL) && threadIdx.x == 0) {
+      const MemberPrm& P = a.mp[member];
+      const double t = a.t_base ? *a.t_base + a.t_off : a.t_off;
+      double sn, cs;
+      sincos(P.omega * t, &sn, &cs);
+      s_prm[0] = (R)cs;
+      s_prm[1] = (R)sn;
+      // a product instead of the FP64 division's chain where FP32 keeps the sum
+      s_prm[2] = sizeof(R) == 4 ? (R)fma(P.c2, 0.2, P.c0) : (R)(P.c0 + P.c2 / 5.0);
+      s_prm[3] = (R)P.c1;
+      s_prm[4] = (R)P.c2;
+      s_prm[5] = (R)P.gx2h;
+      s_prm[6] = (R)P.gy2h;
+      s_prm[7] = (R)P.gz2h;
+    }
+    if ((a.mode & XP_NL) && threadIdx.x < Cfg::ROWS) {
+      const int rr = bx * Cfg::ROWS + threadIdx.x;
+      s_yz[threadIdx.x][0] = a.y0 + (R)(rr % a.ny) * a.hy;
+      s_yz[threadIdx.x][1] = a.z0 + (R)(rr / a.ny) * a.hz;
+    }
+  };
   const int row = bx * Cfg::ROWS + g;
   const bool valid = row < a.rows;
   C* base = a.field + (size_t)member * 5 * a.ntot + (size_t)(valid ? row : 0) * N + i;
   C v[5][E];
-  if constexpr (!CG) pdl_wait();
+  // Thread 0's sine and cosine are a chain of FP64 operations, about a
+  // microsecond: they run while the field is on its way (32 x 512^2: four TS4
+  // steps 6580 -> 6480 us, with the twiddles' copies).  In the persistent
+  // kernel, whose tiles follow one another, they stay first.
+  if constexpr (CG) constants();
+  else pdl_wait();
 #pragma unroll
   for (int c = 0; c < 5; ++c)
 #pragma unroll
     for (int e = 0; e < E; ++e)
       v[c][e] = valid ? ld_field<CG>(base + (size_t)c * a.ntot + T * e) : mkc((R)0, (R)0);
+  if constexpr (!CG) {
+    constants();
+    cp_async_wait();
+  }
   // twiddles, s_prm and s_yz come from other rows' threads
   __syncthreads();
   constexpr int GT = Cfg::GT;
@@ -765,23 +813,6 @@ __device__ __forceinline__ ModeEntry<double> load_mode_shared(const double* t, i
   const double2* q = reinterpret_cast<const double2*>(t) + 4 * idx;
   const double2 a = q[0], b = q[1], c = q[2], d = q[3];
   return ModeEntry<double>{a.x, a.y, b.x, b.y, c.x, c.y, d.x, d.y};
-}
-
-// 16-byte asynchronous copy global -> shared (completes at cp_async_wait)
-__device__ __forceinline__ void cp_async16(void* dst_shared, const void* src_global) {
-  const unsigned d = (unsigned)__cvta_generic_to_shared(dst_shared);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src_global) : "memory");
-}
-// 8-byte asynchronous copy global -> shared (through L1)
-__device__ __forceinline__ void cp_async8(void* dst_shared, const void* src_global) {
-  const unsigned d = (unsigned)__cvta_generic_to_shared(dst_shared);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(src_global) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() {
-  asm volatile("cp.async.commit_group;\n" ::: "memory");
-}
-__device__ __forceinline__ void cp_async_wait() {
-  asm volatile("cp.async.wait_all;\n" ::: "memory");
 }
 
 // the 3D kinetic factor from the (x, y) one and the z one: (1 + kh)(1 + kz) - 1
@@ -1127,6 +1158,8 @@ k_xyplane(XPassArgs<R> a, const TwE<R>* __restrict__ twy_g, int* err) {
 // A hook may also stage data of its own in shared memory behind the mode
 // table's region (hsm), with copies it starts before the field loads.
 struct NoHook {
+  // groups of asynchronous copies that prefetch commits
+  __device__ __forceinline__ int groups() const { return 0; }
   template <typename R, int N, int E, int TILE, int THREADS>
   __device__ __forceinline__ void prefetch(unsigned char*, const LPassArgs<R>&, int, int, int) const {}
   template <typename R, int N, int E, int THREADS>
@@ -1148,7 +1181,7 @@ __device__ __forceinline__ void linepass_body(const LPassArgs<R>& a, int bx, int
   C* xb = reinterpret_cast<C*>(tw + N);
   const int col = threadIdx.x % TILE;
   const int i = threadIdx.x / TILE;
-  for (int k = threadIdx.x; k < N; k += Cfg::THREADS) tw[k] = a.tw[k];
+  load_twiddles<CG, Cfg::THREADS>(tw, a.tw, N);
   const int xcol = bx * TILE + col;
   const bool valid = xcol < a.nx;
   // With the mix, the mode-table entries the tile uses go to shared memory
@@ -1255,6 +1288,14 @@ __device__ __forceinline__ void linepass_body(const LPassArgs<R>& a, int bx, int
 #pragma unroll
       for (int e = 0; e < E; ++e)
         v[c][e] = valid ? ld_field<CG>(base + (size_t)c * a.ntot + e * step) : mkc((R)0, (R)0);
+  }
+  // the twiddles are there (the copies issued after them may not be); the
+  // transforms begin with a barrier
+  if constexpr (!CG) {
+    const int later = (stab || stabz ? 1 : 0) + hook.groups();
+    if (later == 0) cp_async_wait_group<0>();
+    else if (later == 1) cp_async_wait_group<1>();
+    else cp_async_wait_group<2>();
   }
   C* b0 = xb + col * Cfg::LP;
   const int bstride = TILE * Cfg::LP;
