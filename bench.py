@@ -108,7 +108,7 @@ def bytes_per_point_step(dim, scheme, prec, plan=(0, 0, 0)):
 # the sources that define the pass kernels and their launch geometry (the
 # host runtime in sgp_api.cu orchestrates them but does not change a launch's
 # traffic)
-KERNEL_SOURCES = ("sgp_fft.cuh", "sgp_kernels.cuh", "sgp_launch.cuh", "sgp_inst.cu")
+KERNEL_SOURCES = ("sgp_fft.cuh", "sgp_kernels.cuh", "sgp_launch.cuh", "sgp_inst.cu", "sgp_split.cuh", "sgp_fix.cuh")
 
 
 def csrc_hash():

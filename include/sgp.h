@@ -264,8 +264,12 @@ sgp_status sgp_set_graphs(sgp_ctx* ctx, int enable);
  * Kernel variants (FFT tile and radix schedules) and the autotuner.
  * Every pass kernel exists in up to six variants per line length N, and
  * 3D grids have a plane-level variant of the x-pass:
- *   0  default: x-pass CTAs of about 256 threads (rows side by side), line
- *      pass up to 512 threads with TILE >= 4 (FP32) / 2 (FP64) columns;
+ *   0  default: what suits the precision and the number of grid points of
+ *      the batch: passes with the components of a line in threads of their
+ *      own on small FP32 grids, with fixed-point transforms in FP64, one of
+ *      the variants below otherwise; in the groups of an ensemble x-pass
+ *      CTAs of about 256 threads (rows side by side) and line-pass CTAs of up
+ *      to 512 threads with TILE >= 4 (FP32) / 2 (FP64) columns;
  *   1  CTAs of about half the threads (line pass TILE down to 1);
  *   2  CTAs of about a quarter of the threads;
  *   3  FP32 only: for N a power of two the radix-4 plan (4 elements per
