@@ -36,6 +36,14 @@
  *     documented as asynchronous return before the GPU work completes.
  *   - Errors: every call returns an sgp_status; on failure the context keeps
  *     a message readable with sgp_last_error.  No call throws or aborts.
+ *     Passes that bring their tiles in by tensor copies (variant 0 of large
+ *     2D FP32 grids, variants 4 and 5) bound every wait; one that gives up
+ *     is reported as SGP_ETIMEOUT by the next call that hands a result to
+ *     the host or synchronises: sgp_get_state to host memory,
+ *     sgp_get_state_lab, sgp_observables, sgp_step_host, sgp_backward,
+ *     sgp_synchronize, the health check, and the ensemble calls like them.
+ *     The state is then undefined until it is set again.  A copy to device
+ *     memory is asynchronous and cannot report it: sgp_synchronize does.
  *     A context is not thread-safe: one host thread at a time.
  */
 #ifndef SGP_H

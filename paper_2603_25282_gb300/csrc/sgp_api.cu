@@ -344,7 +344,10 @@ struct sgp_ctx {
   // first use) and the word a tile-load wait that gave up sets
   alignas(64) CUtensorMap tmap[3];
   const void* tmap_field[3] = {nullptr, nullptr, nullptr};   // the field a map was made for
+  // set by a tile-load wait that gave up; tiles: such loads have been issued or
+  // captured, so a result handed to the host is preceded by a look at err_dev
   int* err_dev = nullptr;
+  bool tiles = false;
   int var[3] = {0, 0, 0};                        // kernel variant per axis (x-pass, y, z lines)
   // the kernel that variant 0 stands for on each axis (default_kernels), and
   // whether the last work issued on the stream is a pass (which the next pass
@@ -572,6 +575,20 @@ sgp_status get_tables(sgp_ctx* c, double delta, const LinTables** out) {
   return SGP_OK;
 }
 
+// Has a tile-load wait given up since the last look?  For calls that hand a
+// result to the host; the context's streams have been synchronised.
+sgp_status tile_status(sgp_ctx* c) {
+  if (!c->tiles) return SGP_OK;
+  int err = 0;
+  SGP_CUDA(c, cudaMemcpyAsync(&err, c->err_dev, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+  SGP_CUDA(c, cudaStreamSynchronize(c->stream));
+  if (!err) return SGP_OK;
+  SGP_CUDA(c, cudaMemsetAsync(c->err_dev, 0, sizeof(int), c->stream));
+  c->have_state = false;
+  c->adj.valid = false;
+  return fail(c, SGP_ETIMEOUT, "a tile-load wait of a pass gave up; the state is undefined until it is set again");
+}
+
 // ----------------------------------------------------------------------------
 // passes
 // ----------------------------------------------------------------------------
@@ -745,6 +762,7 @@ sgp_status xy_pass_on(sgp_ctx* c, void* field, int mode, double delta, double t_
     c->launches++;
     ProfScope ps(c, PK_X);
     c->chain = false;
+    c->tiles = true;
     SGP_CUDA(c, launch_xyplane(c->n[0], a, (const TwE<R>*)c->tw[1], c->err_dev, c->n[2],
                                 window_members(c), c->stream));
     return SGP_OK;
@@ -812,6 +830,7 @@ sgp_status line_pass_on(sgp_ctx* c, void* field, int axis, int mode, const LinTa
       char* batch_base = (char*)field - (size_t)c->win0 * 5 * c->ntot * c->elem;
       SGP_TRY(ensure_tmap(c, axis, batch_base));
       c->launches++;
+      c->tiles = true;
       ProfScope ps(c, axis == 1 ? PK_Y : PK_Z);
       const bool dep = c->chain && !c->profiling;
       c->chain = true;
@@ -1150,7 +1169,7 @@ sgp_status step_host_impl(sgp_ctx* c, const void* hin, double t0, void* hout, lo
   if (st != SGP_OK) return st;
   for (cudaError_t x : {e, e1, e2, e3, e4})
     if (x != cudaSuccess) return fail(c, SGP_ECUDA, "sgp_step_host: %s", cudaGetErrorString(x));
-  return SGP_OK;
+  return tile_status(c);
 }
 
 // ----------------------------------------------------------------------------
@@ -1748,7 +1767,7 @@ sgp_status state_lab(sgp_ctx* c, void* dst, int on_device) {
                                 c->stream));
   }
   SGP_CUDA(c, cudaStreamSynchronize(c->stream));
-  return SGP_OK;
+  return tile_status(c);
 }
 
 // ----------------------------------------------------------------------------
@@ -1792,6 +1811,7 @@ sgp_status member_mass(sgp_ctx* c, std::vector<double>& out) {
   SGP_CUDA(c, cudaMemcpyAsync(out.data(), c->mass_dev, sizeof(double) * c->batch,
                               cudaMemcpyDeviceToHost, c->stream));
   SGP_CUDA(c, cudaStreamSynchronize(c->stream));
+  SGP_TRY(tile_status(c));
   const double cell = c->h[0] * c->h[1] * (c->dim == 3 ? c->h[2] : 1.0);
   for (double& v : out) v *= cell;
   return SGP_OK;
@@ -2058,6 +2078,7 @@ sgp_status observables(sgp_ctx* c, sgp_obs* out) {
   SGP_CUDA(c, cudaMemcpyAsync(h.data(), c->obs_dev, h.size() * sizeof(double),
                               cudaMemcpyDeviceToHost, c->stream));
   SGP_CUDA(c, cudaStreamSynchronize(c->stream));
+  SGP_TRY(tile_status(c));
   const double cell = c->h[0] * c->h[1] * (c->dim == 3 ? c->h[2] : 1.0);
   bool finite = true;
   for (int m = 0; m < c->batch; ++m) {
@@ -2289,8 +2310,9 @@ sgp_status sgp_get_state(sgp_ctx* c, void* dst, int dst_on_device) {
   SGP_CUDA(c, cudaMemcpyAsync(dst, c->field, bytes,
                               dst_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
                               c->stream));
-  if (!dst_on_device) SGP_CUDA(c, cudaStreamSynchronize(c->stream));
-  return SGP_OK;
+  if (dst_on_device) return SGP_OK;
+  SGP_CUDA(c, cudaStreamSynchronize(c->stream));
+  return tile_status(c);
 }
 
 sgp_status sgp_get_state_lab(sgp_ctx* c, void* dst, int dst_on_device) {
@@ -2397,7 +2419,7 @@ sgp_status sgp_backward(sgp_ctx* c, const void* g_T, int g_T_on_device, void* g_
     SGP_CUDA(c, cudaMemcpyAsync(dparams, r.dp, sizeof(double) * GP_N * c->batch,
                                 cudaMemcpyDeviceToHost, c->stream));
   SGP_CUDA(c, cudaStreamSynchronize(c->stream));
-  return SGP_OK;
+  return tile_status(c);
 }
 
 sgp_status sgp_set_graphs(sgp_ctx* c, int enable) {
@@ -2467,17 +2489,7 @@ sgp_status sgp_synchronize(sgp_ctx* c) {
   if (!c) return SGP_EINVAL;
   DeviceGuard guard(c->device);
   SGP_CUDA(c, cudaStreamSynchronize(c->stream));
-  if (c->err_dev) {
-    int err = 0;
-    SGP_CUDA(c, cudaMemcpy(&err, c->err_dev, sizeof(int), cudaMemcpyDeviceToHost));
-    if (err) {
-      SGP_CUDA(c, cudaMemset(c->err_dev, 0, sizeof(int)));
-      c->have_state = false;
-      return fail(c, SGP_ETIMEOUT, "a tile-load wait of line-pass variant 4 gave up; the state is undefined "
-                                   "until it is set again");
-    }
-  }
-  return SGP_OK;
+  return tile_status(c);
 }
 
 long long sgp_launch_count(const sgp_ctx* c) { return c ? c->launches : 0; }
@@ -2612,6 +2624,17 @@ sgp_status efail(sgp_ens* e, sgp_status s, const char* fmt, ...) {
 void ens_free_graphs(sgp_ens* e) {
   for (auto& g : e->graphs) cudaGraphExecDestroy(g.exec);
   e->graphs.clear();
+}
+
+// tile_status of every group (the ensemble's stream has been synchronised)
+sgp_status ens_tile_status(sgp_ens* e) {
+  sgp_status st = SGP_OK;
+  for (size_t g = 0; g < e->groups.size(); ++g) {
+    const sgp_status s = tile_status(e->groups[g]);
+    if (s == SGP_ETIMEOUT) e->have_state = false;
+    if (s != SGP_OK && st == SGP_OK) st = efail(e, s, "group %zu: %s", g, e->groups[g]->err.c_str());
+  }
+  return st;
 }
 
 // Issue `steps` steps of every group: group g on stream s(g).
@@ -3091,7 +3114,7 @@ sgp_status sgp_ensemble_get_member_state(sgp_ens* e, int member, void* dst, int 
                                    e->stream);
   if (ce == cudaSuccess && !dst_on_device) ce = cudaStreamSynchronize(e->stream);
   if (ce != cudaSuccess) return efail(e, SGP_ECUDA, "copy: %s", cudaGetErrorString(ce));
-  return SGP_OK;
+  return dst_on_device ? SGP_OK : ens_tile_status(e);
 }
 
 sgp_status sgp_ensemble_step_host(sgp_ens* e, const void* const* host_in, double t0,
@@ -3189,7 +3212,7 @@ sgp_status sgp_ensemble_step_host(sgp_ens* e, const void* const* host_in, double
   if (st != SGP_OK) return st;
   if (ce == cudaSuccess) ce = cs;
   if (ce != cudaSuccess) return efail(e, SGP_ECUDA, "copy out: %s", cudaGetErrorString(ce));
-  return SGP_OK;
+  return ens_tile_status(e);
 }
 
 sgp_status sgp_ensemble_step(sgp_ens* e, long long nsteps, double dt, int scheme) {
@@ -3244,7 +3267,7 @@ sgp_status sgp_ensemble_synchronize(sgp_ens* e) {
   DeviceGuard guard(e->device);
   cudaError_t ce = cudaStreamSynchronize(e->stream);
   if (ce != cudaSuccess) return efail(e, SGP_ECUDA, "%s", cudaGetErrorString(ce));
-  return SGP_OK;
+  return ens_tile_status(e);
 }
 
 long long sgp_ensemble_launch_count(const sgp_ens* e) { return e ? e->launches : 0; }
