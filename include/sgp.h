@@ -320,8 +320,9 @@ sgp_status sgp_get_plan(const sgp_ctx* ctx, int* variants);
  * CUDA events on the context stream; keep the fastest (a higher-numbered
  * variant must be at least 1.5% faster to replace a lower one).  The state
  * and the time are not changed.  Results are cached per process by
- * (device, precision, grid, batch); a cached plan is reused unless flags
- * has SGP_TUNE_FORCE or ms_out is given.  ms_out (may be NULL): 3 x 7
+ * (device, precision, grid, batch), apart for contexts and for the groups of
+ * ensembles, whose variant 0 is another kernel; a cached plan is reused
+ * unless flags has SGP_TUNE_FORCE or ms_out is given.  ms_out (may be NULL): 3 x 7
  * doubles, ms per step of [axis][variant], -1 where the variant or axis
  * does not exist, for variant 4 of the x-pass (which is variant 1) and for
  * variant 6 of the line passes (which is variant 2).

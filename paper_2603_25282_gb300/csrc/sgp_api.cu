@@ -1896,8 +1896,9 @@ sgp_status use_variant(sgp_ctx* c, int a, int v) {
   return SGP_OK;
 }
 
-// process-wide results of the autotuner, keyed by device, precision, grid
-// and batch
+// process-wide results of the autotuner, keyed by device, precision, grid,
+// batch and what variant 0 stands for on each axis (the groups of an ensemble
+// time the plain kernels in its place: their plans are not a context's)
 std::map<std::string, std::vector<int>>& tune_cache() {
   static std::map<std::string, std::vector<int>> m;
   return m;
@@ -1905,8 +1906,8 @@ std::map<std::string, std::vector<int>>& tune_cache() {
 
 std::string tune_key(const sgp_ctx* c) {
   char b[160];
-  snprintf(b, sizeof b, "%d:%d:%d:%d:%d:%d:%d", c->device, c->prec, c->dim, c->n[0], c->n[1],
-           c->n[2], c->batch);
+  snprintf(b, sizeof b, "%d:%d:%d:%d:%d:%d:%d:%d:%d:%d", c->device, c->prec, c->dim, c->n[0], c->n[1],
+           c->n[2], c->batch, c->def[0], c->def[1], c->def[2]);
   return b;
 }
 
