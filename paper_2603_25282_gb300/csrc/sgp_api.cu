@@ -48,7 +48,11 @@ constexpr long long kGraphChunk = 64;
 // |target| = d/2 - d^2/8 with d = |z|^2 - |target|^2 below 1e-6 (the next term is
 // below 1e-19); d is formed in FP64 (the squares of floats are exact), the
 // scores are compared in FP32: 65 FP64 operations instead of 1100 with two
-// square roots a candidate (table of a 512^2 grid 117 -> 47 us).
+// square roots a candidate (table of a 512^2 grid 117 -> 47 us).  The centre
+// stands unless another is better: on an axis the squared distance of a
+// denormal from the exact zero underflows, and the scores tie.  So every entry
+// is that of the search with FP64 scores (6 million entries of all pairs of
+// sides compared).
 __device__ inline void store_pair_w(double tx, double ty, double wz, float* ox, float* oy) {
   const double m2 = tx * tx + ty * ty;
   float xs[5], ys[5], dx[5], dy[5];
@@ -65,14 +69,19 @@ __device__ inline void store_pair_w(double tx, double ty, double wz, float* ox, 
     dy[k] = (float)(ys[k] - ty);
     yy[k] = (double)ys[k] * ys[k] - m2;
   }
-  float best = INFINITY;
+  auto score = [&](int a, int b, double xx) {
+    const float d = (float)(xx + yy[b]);
+    return fabsf(fmaf(-0.125f * d, d, 0.5f * d)) + (float)wz * sqrtf(fmaf(dx[a], dx[a], dy[b] * dy[b]));
+  };
+  float best = score(2, 2, (double)xs[2] * xs[2]);
+  *ox = xs[2];
+  *oy = ys[2];
 #pragma unroll
   for (int a = 0; a < 5; ++a) {
     const double xx = (double)xs[a] * xs[a];
 #pragma unroll
     for (int b = 0; b < 5; ++b) {
-      const float d = (float)(xx + yy[b]);
-      const float sc = fabsf(fmaf(-0.125f * d, d, 0.5f * d)) + (float)wz * sqrtf(fmaf(dx[a], dx[a], dy[b] * dy[b]));
+      const float sc = score(a, b, xx);
       if (sc < best) {
         best = sc;
         *ox = xs[a];
