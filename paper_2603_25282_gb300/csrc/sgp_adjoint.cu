@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(kXAdjThreads, 2) k_xadj(XAdjArgs<R> a) {
     const MemberPrm& P = a.mp[member];
     NLAdjPrm<R> q;
     q.d = (R)a.delta;
-    q.c0p = (R)(P.c0 + P.c2 / 5.0);
+    q.c0p = coupling<R>(P);
     q.c1 = (R)P.c1;
     q.c2 = (R)P.c2;
     q.tdgg = (R)(s_rot[2] * 2.0 * (P.gx2h - P.gy2h));

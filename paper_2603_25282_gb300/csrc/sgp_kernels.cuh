@@ -36,6 +36,14 @@ struct MemberPrm {
   double omega, gamma, c0, c1, c2;
   double gx2h, gy2h, gz2h;   // gx^2/2, gy^2/2, gz^2/2 (gz2h = 0 in 2D)
 };
+
+// c0 + c2/5, the density's coupling in the nonlinear flow, as every kernel of a
+// precision forms it (variants that agree bit for bit need the same sum).  FP32
+// keeps 24 bits of it: a product there instead of the FP64 division's chain.
+template <typename R>
+__device__ __forceinline__ R coupling(const MemberPrm& P) {
+  return sizeof(R) == 4 ? (R)fma(P.c2, 0.2, P.c0) : (R)(P.c0 + P.c2 / 5.0);
+}
 // line-pass mode bits
 enum { LP_FWD = 1, LP_MIX = 2, LP_INV = 4 };
 
@@ -573,8 +581,7 @@ __device__ __forceinline__ void xpass_body(const XPassArgs<R>& a, int bx, int me
       sincos(P.omega * t, &sn, &cs);
       s_prm[0] = (R)cs;
       s_prm[1] = (R)sn;
-      // a product instead of the FP64 division's chain where FP32 keeps the sum
-      s_prm[2] = sizeof(R) == 4 ? (R)fma(P.c2, 0.2, P.c0) : (R)(P.c0 + P.c2 / 5.0);
+      s_prm[2] = coupling<R>(P);
       s_prm[3] = (R)P.c1;
       s_prm[4] = (R)P.c2;
       s_prm[5] = (R)P.gx2h;
@@ -676,7 +683,7 @@ __global__ void __launch_bounds__(kXWideThreads, 2) k_xpass_wide(XPassArgs<R> a)
     sincos(P.omega * t, &sn, &cs);
     s_prm[0] = (R)cs;
     s_prm[1] = (R)sn;
-    s_prm[2] = (R)(P.c0 + P.c2 / 5.0);
+    s_prm[2] = coupling<R>(P);
     s_prm[3] = (R)P.c1;
     s_prm[4] = (R)P.c2;
     s_prm[5] = (R)P.gx2h;
@@ -1049,7 +1056,7 @@ k_xyplane(XPassArgs<R> a, const TwE<R>* __restrict__ twy_g, int* err) {
     sincos(P.omega * t, &sn, &cs);
     s_prm[0] = (R)cs;
     s_prm[1] = (R)sn;
-    s_prm[2] = (R)(P.c0 + P.c2 / 5.0);
+    s_prm[2] = coupling<R>(P);
     s_prm[3] = (R)P.c1;
     s_prm[4] = (R)P.c2;
     s_prm[5] = (R)P.gx2h;

@@ -93,7 +93,7 @@ k_xsplit(XPassArgs<R> a) {
     sincos(P.omega * t, &sn, &cs);
     s_prm[0] = (R)cs;
     s_prm[1] = (R)sn;
-    s_prm[2] = (R)(P.c0 + P.c2 / 5.0);
+    s_prm[2] = coupling<R>(P);
     s_prm[3] = (R)P.c1;
     s_prm[4] = (R)P.c2;
     s_prm[5] = (R)P.gx2h;
@@ -370,7 +370,7 @@ k_xadj_split(XAdjArgs<R> a) {
     const MemberPrm& P = a.mp[member];
     NLAdjPrm<R> q;
     q.d = (R)a.delta;
-    q.c0p = (R)(P.c0 + P.c2 / 5.0);
+    q.c0p = coupling<R>(P);
     q.c1 = (R)P.c1;
     q.c2 = (R)P.c2;
     q.tdgg = (R)(s_rot[2] * 2.0 * (P.gx2h - P.gy2h));
