@@ -88,7 +88,7 @@ typedef void* (*sgp_alloc_fn)(size_t bytes, int device, void* stream, void* user
 typedef void (*sgp_free_fn)(void* ptr, int device, void* stream, void* user);
 
 /* Flags of sgp_autotune. */
-enum { SGP_TUNE_FORCE = 1 };
+enum { SGP_TUNE_FORCE = 1, SGP_TUNE_ALL = 2 };
 
 /* Substep kinds for sgp_substep. */
 typedef enum { SGP_SUB_NONLINEAR = 0, SGP_SUB_LINEAR = 1 } sgp_substep_kind;
@@ -270,14 +270,15 @@ sgp_status sgp_set_graphs(sgp_ctx* ctx, int enable);
 
 /* ---------------------------------------------------------------------
  * Kernel variants (FFT tile and radix schedules) and the autotuner.
- * Every pass kernel exists in up to six variants per line length N, and
+ * Every pass kernel exists in up to seven variants per line length N, and
  * 3D grids have a plane-level variant of the x-pass:
  *   0  default: what suits the precision and the number of grid points of
  *      the batch: passes with the components of a line in threads of their
  *      own on small FP32 grids, with fixed-point transforms in FP64, one of
- *      the variants below otherwise; in the groups of an ensemble x-pass
- *      CTAs of about 256 threads (rows side by side) and line-pass CTAs of up
- *      to 512 threads with TILE >= 4 (FP32) / 2 (FP64) columns;
+ *      the variants below otherwise; in the groups of an ensemble variant 7.
+ *      The choice goes by the points of the whole batch, so a member's low
+ *      bits may differ between a run alone and a run in a batch (or a shard
+ *      of one): those of plans without variant 0 on any axis do not;
  *   1  CTAs of about half the threads (line pass TILE down to 1);
  *   2  CTAs of about a quarter of the threads;
  *   3  FP32 only: for N a power of two the radix-4 plan (4 elements per
@@ -295,7 +296,11 @@ sgp_status sgp_set_graphs(sgp_ctx* ctx, int enable);
  *      observables) are those of variant 1;
  *   6  x-pass: CTAs of variant 2's rows with the nonlinear flow shared by
  *      256 threads (for small grids, whose CTAs are few, each thread takes
- *      fewer points through the flow); line pass: the same as variant 2.
+ *      fewer points through the flow); line pass: the same as variant 2;
+ *   7  the plain kernels at any size: x-pass CTAs of about 256 threads (rows
+ *      side by side), line-pass CTAs of up to 512 threads with TILE >= 4
+ *      (FP32) / 2 (FP64) columns.  A gradient's passes go by the size like
+ *      variant 0, but with variant 7 on some axis they are the plain ones.
  * A plan is one variant per axis (x-pass, y lines, z lines).  Variants
  * compute the same transforms with different rounding (variant 3 has a
  * different radix plan), so results agree to rounding, not bit for bit;
@@ -322,10 +327,12 @@ sgp_status sgp_get_plan(const sgp_ctx* ctx, int* variants);
  * and the time are not changed.  Results are cached per process by
  * (device, precision, grid, batch), apart for contexts and for the groups of
  * ensembles, whose variant 0 is another kernel; a cached plan is reused
- * unless flags has SGP_TUNE_FORCE or ms_out is given.  ms_out (may be NULL): 3 x 7
- * doubles, ms per step of [axis][variant], -1 where the variant or axis
+ * unless flags has SGP_TUNE_FORCE or ms_out is given.  ms_out (may be NULL):
+ * 3 x 7 doubles, ms per step of [axis][variant], -1 where the variant or axis
  * does not exist, for variant 4 of the x-pass (which is variant 1) and for
- * variant 6 of the line passes (which is variant 2).
+ * variant 6 of the line passes (which is variant 2); variant 7 is then not
+ * among the choices.  With SGP_TUNE_ALL in flags ms_out is 3 x 8 doubles and
+ * it is.  Variants that stand for the same kernel are timed once.
  * Synchronises.  Allocates one field-sized scratch buffer
  * for the duration of the call.  Errors: SGP_EINVAL for a NULL ctx or reps
  * outside [1, 1000]; SGP_ENOMEM / SGP_ECUDA for the scratch or a launch. */

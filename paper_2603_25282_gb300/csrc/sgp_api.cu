@@ -707,7 +707,8 @@ void default_kernels(sgp_ctx* c, bool legacy) {
 }
 
 // the kernel an axis runs: its variant, or what variant 0 stands for
-int axis_kernel(const sgp_ctx* c, int a) { return c->var[a] == 0 ? c->def[a] : c->var[a]; }
+int kernel_of(const sgp_ctx* c, int a, int v) { return v == 0 ? c->def[a] : v == 7 ? 0 : v; }
+int axis_kernel(const sgp_ctx* c, int a) { return kernel_of(c, a, c->var[a]); }
 
 template <typename R>
 XPassArgs<R> x_args(const sgp_ctx* c, void* field, int mode, double delta, double t_off) {
@@ -1244,11 +1245,12 @@ sgp_status record_steps(sgp_ctx* c, long long nsteps, double dt, int scheme, lon
 // Rows of the parameter partials per member: one per CTA of the adjoint
 // x-pass, then one per CTA of the line pass that holds the full transform
 // (y lines in 2D, z lines in 3D).
-// On grids whose passes are the FP32 component-parallel ones, a gradient's are too.
+// On grids whose passes are the FP32 component-parallel ones, a gradient's are
+// too, unless the plan has the plain kernels on some axis (variant 7).
 bool adj_split(const sgp_ctx* c) {
   if (c->prec != SGP_F32) return false;
   for (int a = 0; a < c->dim; ++a)
-    if (c->def[a] != kSplitPass) return false;
+    if (c->def[a] != kSplitPass || c->var[a] == 7) return false;
   return true;
 }
 template <typename R>
@@ -1926,11 +1928,12 @@ std::string tune_key(const sgp_ctx* c) {
 // warm-up step: the data stay a physical state, so the nonlinear flow takes
 // its usual branches, and the pass interplay of a real step is included.  A
 // variant replaces an earlier (lower-numbered) one only when it is at least
-// 1.5% faster, so near-ties resolve the same way run to run.  ms_out[3][7]:
-// ms per step with that variant (-1 where a variant does not exist or the
-// axis is absent).
+// 1.5% faster, so near-ties resolve the same way run to run.  A variant whose
+// kernel an earlier one has already run takes that one's time.
+// ms_out[3][cols]: ms per step with that variant (-1 where a variant does not
+// exist or the axis is absent); variants from cols on are left out.
 template <typename R>
-sgp_status autotune_impl(sgp_ctx* c, int reps, double* ms_out) {
+sgp_status autotune_impl(sgp_ctx* c, int reps, int cols, double* ms_out) {
   const size_t sb = state_bytes(c);
   void* scratch = nullptr;
   SGP_CUDA(c, cudaStreamSynchronize(c->stream));
@@ -1944,14 +1947,21 @@ sgp_status autotune_impl(sgp_ctx* c, int reps, double* ms_out) {
   cudaEventCreate(&e1);
   int best[3] = {c->var[0], c->var[1], c->var[2]};
   if (ms_out)
-    for (int k = 0; k < 3 * kVariants; ++k) ms_out[k] = -1.0;
+    for (int k = 0; k < 3 * cols; ++k) ms_out[k] = -1.0;
   for (int a = 0; a < c->dim && st == SGP_OK; ++a) {
-    double best_ms = -1.0;
-    for (int v = 0; v < kVariants && st == SGP_OK; ++v) {
+    double best_ms = -1.0, took[kVariants];
+    std::fill(took, took + kVariants, -1.0);
+    for (int v = 0; v < cols && st == SGP_OK; ++v) {
       if (!axis_variant_ok(c, a, v)) continue;
       if (a == 0 && v == 4) continue;     // the x-pass of variant 4 is variant 1
       if (a != 0 && v == 6) continue;     // the line pass of variant 6 is variant 2
       if (v == 4 && !tensor_map_encoder()) continue;
+      for (int u = 0; u < v && took[v] < 0.0; ++u)
+        if (took[u] >= 0.0 && kernel_of(c, a, u) == kernel_of(c, a, v)) took[v] = took[u];
+      if (took[v] >= 0.0) {
+        if (ms_out) ms_out[a * cols + v] = took[v];
+        continue;
+      }
       st = use_variant(c, a, v);
       if (st != SGP_OK) break;
       c->launches++;
@@ -1968,8 +1978,8 @@ sgp_status autotune_impl(sgp_ctx* c, int reps, double* ms_out) {
       }
       float ms = 0.f;
       cudaEventElapsedTime(&ms, e0, e1);
-      const double avg = ms / reps;
-      if (ms_out) ms_out[a * kVariants + v] = avg;
+      const double avg = took[v] = ms / reps;
+      if (ms_out) ms_out[a * cols + v] = avg;
       if (best_ms < 0.0 || avg < 0.985 * best_ms) {
         best_ms = avg;
         best[a] = v;
@@ -2472,8 +2482,10 @@ sgp_status sgp_autotune(sgp_ctx* c, int reps, int flags, double* ms_out) {
       return SGP_OK;
     }
   }
-  return c->prec == SGP_F32 ? autotune_impl<float>(c, reps, ms_out)
-                            : autotune_impl<double>(c, reps, ms_out);
+  // a caller's table of 7 columns has no place for variant 7
+  const int cols = !ms_out || (flags & SGP_TUNE_ALL) ? kVariants : 7;
+  return c->prec == SGP_F32 ? autotune_impl<float>(c, reps, cols, ms_out)
+                            : autotune_impl<double>(c, reps, cols, ms_out);
 }
 
 sgp_status sgp_substep(sgp_ctx* c, int kind, double delta) {

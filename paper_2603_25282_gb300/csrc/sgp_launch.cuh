@@ -53,7 +53,9 @@ inline bool supported_n(int n) {
 //   6  x-pass: the rows of geometry 2 with the nonlinear flow shared by the
 //      256 threads of the CTA (k_xpass_wide; for small grids, whose CTAs
 //      are few); line pass: the same as variant 2
-constexpr int kVariants = 7;
+//   7  the default geometry itself, whatever the size (variant 0 of the groups
+//      of an ensemble): a member's result does not depend on the batch
+constexpr int kVariants = 8;
 
 template <typename R, int N, int V>
 constexpr int variant_elems() {
@@ -62,7 +64,7 @@ constexpr int variant_elems() {
 // geometry of variant V for the x-pass (PART 0) and the line pass (PART 1)
 template <int N, int V, int PART>
 constexpr int variant_geom() {
-  return V == 3 ? (N % 3 == 0 ? 1 + PART : 0) : (V == 4 || V == 5) ? 1 : V == 6 ? 2 : V;
+  return V == 3 ? (N % 3 == 0 ? 1 + PART : 0) : (V == 4 || V == 5) ? 1 : V == 6 ? 2 : V == 7 ? 0 : V;
 }
 
 // Does variant V exist for line length N (prec_bytes 4 or 8)?
@@ -132,8 +134,8 @@ cudaError_t prepare_xpass_wide(int N);
 
 // x-pass variants 4 and 5 are variant 1 (variant 5's plane pass has its own
 // entry point) and variant 6 has the geometry of variant 2 (its own kernel,
-// dispatched first); the line pass has its own variant 4 and takes variant
-// 2 for 6
+// dispatched first), variant 7 is variant 0; the line pass has its own variant
+// 4 and takes variant 2 for 6
 #define SGP_VARIANT_SWITCH_X(V, CALL, FAIL)                  \
   switch (V) {                                               \
     case 0: return CALL(0);                                  \
@@ -147,6 +149,7 @@ cudaError_t prepare_xpass_wide(int N);
       if constexpr (sizeof(R) == 4) return CALL(1);          \
       return FAIL;                                           \
     case 6: return CALL(2);                                  \
+    case 7: return CALL(0);                                  \
     default: return FAIL;                                    \
   }
 #define SGP_VARIANT_SWITCH(V, CALL, FAIL)                    \
@@ -158,6 +161,7 @@ cudaError_t prepare_xpass_wide(int N);
       if constexpr (sizeof(R) == 4) return CALL(3);          \
       return FAIL;                                           \
     case 6: return CALL(2);                                  \
+    case 7: return CALL(0);                                  \
     default: return FAIL;                                    \
   }
 

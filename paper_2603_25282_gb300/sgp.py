@@ -284,8 +284,8 @@ def step_host(ctx, src, t0, dst, nsteps, dt, scheme, chunks, dtype):
     return dst
 
 
-SGP_TUNE_FORCE = 1
-N_VARIANTS = 7
+SGP_TUNE_FORCE, SGP_TUNE_ALL = 1, 2
+N_VARIANTS = 8
 
 
 def variant_exists(prec, n, variant):
@@ -309,7 +309,7 @@ def autotune(ctx, reps=20, force=False, timings=False):
     """sgp_autotune; returns the plan, and with timings=True also the
     [axis][variant] ms per launch (None where absent)."""
     ms = (ctypes.c_double * (3 * N_VARIANTS))() if timings else None
-    _check(lib().sgp_autotune(ctx, int(reps), SGP_TUNE_FORCE if force else 0, ms), ctx)
+    _check(lib().sgp_autotune(ctx, int(reps), (SGP_TUNE_FORCE if force else 0) | SGP_TUNE_ALL, ms), ctx)
     plan = get_plan(ctx)
     if not timings:
         return plan
