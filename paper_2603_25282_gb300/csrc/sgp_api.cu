@@ -667,43 +667,15 @@ bool plane_ok(const sgp_ctx* c) {
 // which has no plane pass.
 bool plane_pass(const sgp_ctx* c) { return c->var[0] == 5 && !c->rec; }
 
-// What variant 0 of an axis stands for, by the size of the whole batch (pts
-// grid points), the precision and the line length; measured per TS2 step on
-// the GB300 (plain variant 0 -> the choice, us):
-//   component-parallel passes for grids of few lines: FP32 2D up to 192 Ki
-//     points (64^2 22 -> 5, 256^2 32 -> 10, 384^2 44 -> 27; from 256 Ki points
-//     the others are ahead: 4 x 256^2 27 against 33), 3D below 128 Ki (48^3
-//     35 -> 28; 64 x 64 x 32 28 against 30);
-//   FP64 everywhere (fixed-point transforms, sgp_fix.cuh: 64^2 229 -> 50, 8 x
-//     512^2 5300 -> 2500, 128^3 5510 -> 2610), with one line per CTA while that
-//     gives no more than four CTAs an SM;
-//   FP32 2D otherwise: TMA tiles for the y-lines (768^2 104 -> 90 with x-pass
-//     geometry 1), geometry 1 for the x-pass except at 512 (16 x 256^2 75 ->
-//     72, 4 x 1024^2 367 -> 357, but 16 x 512^2 281 -> 288);
-//   FP32 3D otherwise: geometry 1 on every axis (128^3 230 -> 190).
-// With legacy (the groups of an ensemble, which stay comparable to the
-// persistent kernel bit for bit) variant 0 is the plain kernel.
-constexpr int kSplitPass = 100, kSplitMany = 101;
 PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder();
 
+// The kernels of variant 0.  With legacy (the groups of an ensemble, which stay
+// comparable to the persistent kernel bit for bit) they are the plain ones.
 void default_kernels(sgp_ctx* c, bool legacy) {
-  const long long pts = c->ntot * c->batch;
-  for (int a = 0; a < c->dim; ++a) {
-    c->def[a] = 0;
-    if (legacy) continue;
-    if (c->prec == SGP_F32) {
-      if (split_exists<float>(c->n[a]) && pts <= (c->dim == 2 ? 3LL << 16 : (1LL << 17) - 1))
-        c->def[a] = kSplitPass;
-      else if (c->dim == 3)
-        c->def[a] = 1;
-      else if (a == 0)
-        c->def[a] = c->n[0] == 512 ? 0 : 1;
-      else
-        c->def[a] = tensor_map_encoder() ? 4 : 1;
-    } else if (split_exists<double>(c->n[a])) {
-      c->def[a] = pts / c->n[a] > 4 * 152 ? kSplitMany : kSplitPass;
-    }
-  }
+  for (int a = 0; a < c->dim; ++a)
+    c->def[a] = legacy ? 0
+                       : default_kernel(c->prec == SGP_F32 ? 4 : 8, c->dim, c->n, c->batch, a,
+                                        tensor_map_encoder() != nullptr);
 }
 
 // the kernel an axis runs: its variant, or what variant 0 stands for

@@ -162,11 +162,6 @@ cudaError_t launch_fix_twiddles(int N, FixTw* out, cudaStream_t s) {
 }
 
 template <>
-bool split_exists<double>(int N) {
-  return supported_n(N);
-}
-
-template <>
 cudaError_t prepare_xsplit<double>(int N, bool many) {
 #define SGP_CASE(NN) case NN: return many ? xfix_prepare<NN, fix_lines<NN>(true)>() : xfix_prepare<NN, 1>();
   SGP_SWITCH(SGP_CASE, cudaErrorInvalidValue)

@@ -34,8 +34,8 @@ inline bool supported_n(int n) {
 // chooses from):
 //   0  default geometry (x-pass: about 256 threads per CTA; line pass: up
 //      to 512 threads, TILE >= 4 FP32 / 2 FP64 columns) and radix plan
-//      (a context takes for it what suits its size: default_kernels in
-//      sgp_api.cu, with the component-parallel passes of sgp_split.cuh)
+//      (a context takes for it what suits its size: default_kernel below,
+//      with the component-parallel passes of sgp_split.cuh)
 //   1  CTAs of about half the threads (line pass: TILE down to 1)
 //   2  CTAs of about a quarter of the threads
 //   3  FP32 only.  N a power of two: radix-4 plan (4 elements per thread
@@ -216,6 +216,31 @@ inline cudaError_t launch_linepass(int N, int V, const LPassArgs<R>& a, int plan
 }
 #undef SGP_VARIANT_SWITCH
 #undef SGP_VARIANT_SWITCH_X
+
+// What variant 0 of an axis stands for, by the size of the whole batch (pts
+// grid points), the precision and the line length; measured per TS2 step on
+// the GB300 (plain variant 0 -> the choice, us):
+//   component-parallel passes for grids of few lines: FP32 2D up to 192 Ki
+//     points (64^2 22 -> 5, 256^2 32 -> 10, 384^2 44 -> 27; from 256 Ki points
+//     the others are ahead: 4 x 256^2 27 against 33), 3D below 128 Ki (48^3
+//     35 -> 28; 64 x 64 x 32 28 against 30);
+//   FP64 everywhere (fixed-point transforms, sgp_fix.cuh: 64^2 229 -> 50, 8 x
+//     512^2 5300 -> 2500, 128^3 5510 -> 2610), with one line per CTA while that
+//     gives no more than four CTAs an SM;
+//   FP32 2D otherwise: TMA tiles for the y-lines (768^2 104 -> 90 with x-pass
+//     geometry 1), geometry 1 for the x-pass except at 512 (16 x 256^2 75 ->
+//     72, 4 x 1024^2 367 -> 357, but 16 x 512^2 281 -> 288);
+//   FP32 3D otherwise: geometry 1 on every axis (128^3 230 -> 190).
+constexpr int kSplitPass = 100, kSplitMany = 101;
+
+inline int default_kernel(int prec_bytes, int dim, const int* n, int batch, int a, bool tensor_maps) {
+  const long long pts = (long long)n[0] * n[1] * (dim == 3 ? n[2] : 1) * batch;
+  if (prec_bytes == 8) return pts / n[a] > 4 * 152 ? kSplitMany : kSplitPass;
+  if (pts <= (dim == 2 ? 3LL << 16 : (1LL << 17) - 1)) return kSplitPass;
+  if (dim == 3) return 1;
+  if (a == 0) return n[0] == 512 ? 0 : 1;
+  return tensor_maps ? 4 : 1;
+}
 
 // Observables kernels (default geometry only).
 template <typename R>

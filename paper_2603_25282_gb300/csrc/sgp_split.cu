@@ -106,11 +106,6 @@ cudaError_t ladj_n(const LPassArgs<float>& a, const AdjHook<float>& h, int plane
   }
 
 template <>
-bool split_exists<float>(int N) {
-  return supported_n(N);
-}
-
-template <>
 int split_elems_rt<float>(int N) {
 #define SGP_CASE(NN) case NN: return split_elems<float, NN>();
   SGP_SWITCH(SGP_CASE, 0)

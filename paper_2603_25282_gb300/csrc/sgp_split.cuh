@@ -432,7 +432,6 @@ constexpr int split_elems() { return N % 3 == 0 ? 12 : 8; }
 // are those of sgp_fix.cuh (sgp_fix.cu).  dependent: the launch may begin
 // while the pass before it on the stream is at work.  many (FP64): enough
 // lines for CTAs of several.
-template <typename R> bool split_exists(int N);
 template <typename R> int split_elems_rt(int N);
 template <typename R> cudaError_t prepare_xsplit(int N, bool many);
 template <typename R> cudaError_t prepare_lsplit(int N, bool many);
