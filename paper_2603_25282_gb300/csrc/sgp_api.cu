@@ -362,6 +362,7 @@ struct sgp_ctx {
   // whether the last work issued on the stream is a pass (which the next pass
   // may follow as a dependent launch)
   int def[3] = {0, 0, 0};
+  int sms = 1;                                   // of the device
   // passes issued one by one carry the time themselves: the start of their run
   bool own_time = false;
   double run_t0 = 0.0;
@@ -675,7 +676,7 @@ void default_kernels(sgp_ctx* c, bool legacy) {
   for (int a = 0; a < c->dim; ++a)
     c->def[a] = legacy ? 0
                        : default_kernel(c->prec == SGP_F32 ? 4 : 8, c->dim, c->n, c->batch, a,
-                                        tensor_map_encoder() != nullptr);
+                                        tensor_map_encoder() != nullptr, c->sms);
 }
 
 // the kernel an axis runs: its variant, or what variant 0 stands for
@@ -2184,6 +2185,8 @@ sgp_status sgp_create_grid(int dim, const int* n, const double* L, int batch, in
                         : (a == 0 ? prepare_xpass<double>(c->n[a]) : prepare_linepass<double>(c->n[a]));
     if (e != cudaSuccess) return bail(SGP_ECUDA, "kernel attributes", e);
   }
+  if ((e = cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, device)) != cudaSuccess)
+    return bail(SGP_ECUDA, "device attribute", e);
   default_kernels(c, false);
   for (int a = 0; a < dim && e == cudaSuccess; ++a) {
     const int v = c->def[a];

@@ -228,17 +228,32 @@ inline cudaError_t launch_linepass(int N, int V, const LPassArgs<R>& a, int plan
 //     512^2 5300 -> 2500, 128^3 5510 -> 2610), with one line per CTA while that
 //     gives no more than four CTAs an SM;
 //   FP32 2D otherwise: TMA tiles for the y-lines (768^2 104 -> 90 with x-pass
-//     geometry 1), geometry 1 for the x-pass except at 512 (16 x 256^2 75 ->
-//     72, 4 x 1024^2 367 -> 357, but 16 x 512^2 281 -> 288);
+//     geometry 1), for the x-pass geometry 1 or that of long_row_geometry;
 //   FP32 3D otherwise: geometry 1 on every axis (128^3 230 -> 190).
 constexpr int kSplitPass = 100, kSplitMany = 101;
 
-inline int default_kernel(int prec_bytes, int dim, const int* n, int batch, int a, bool tensor_maps) {
+// x-pass geometry of FP32 rows of 512 or 1024 points, by the last wave: CTAs of
+// 256 threads (geometry 0) cost less than twice as many of 128 (geometry 1)
+// where they do not end later, that is where halving them saves no part of a
+// wave of one CTA an SM; 1024 points past two CTAs an SM take geometry 1.  us per
+// TS2 step with geometry 0 and 1, rows of 512: 512 rows 26.1 and 27.0, 640 38.5
+// and 35.5, 1024 39.7 and 41.5, 1408 59.2 and 56.8, 2048 75.4 and 73.9, 4096
+// 135.9 and 138.0; of 1024: 384 45.0 and 39.7, 512 45.6 and 47.0, 2048 156 and
+// 150.  Shorter rows are within 1% at 256 and ahead with geometry 1 below (64:
+// 23.8 and 22.9), those of 3*2^k ahead with it or level.
+inline int long_row_geometry(int nx, long long rows, int sms) {
+  const long long c0 = (rows + xpass_geom<float>(nx, 0).rows_or_tile - 1) / xpass_geom<float>(nx, 0).rows_or_tile;
+  const long long c1 = (rows + xpass_geom<float>(nx, 1).rows_or_tile - 1) / xpass_geom<float>(nx, 1).rows_or_tile;
+  const bool level = 2 * ((c0 + sms - 1) / sms) <= (c1 + sms - 1) / sms;
+  return level && (nx <= 512 || c0 <= 2LL * sms) ? 0 : 1;
+}
+
+inline int default_kernel(int prec_bytes, int dim, const int* n, int batch, int a, bool tensor_maps, int sms) {
   const long long pts = (long long)n[0] * n[1] * (dim == 3 ? n[2] : 1) * batch;
-  if (prec_bytes == 8) return pts / n[a] > 4 * 152 ? kSplitMany : kSplitPass;
+  if (prec_bytes == 8) return pts / n[a] > 4LL * sms ? kSplitMany : kSplitPass;
   if (pts <= (dim == 2 ? 3LL << 16 : (1LL << 17) - 1)) return kSplitPass;
   if (dim == 3) return 1;
-  if (a == 0) return n[0] == 512 ? 0 : 1;
+  if (a == 0) return n[0] >= 512 && n[0] % 3 != 0 ? long_row_geometry(n[0], pts / n[0], sms) : 1;
   return tensor_maps ? 4 : 1;
 }
 

@@ -1,0 +1,53 @@
+"""Where variant 0 changes its kernels, the choice is not behind the plain ones:
+time per step against the x-pass geometries that the rule chooses between.
+
+Two runs of one kernel differ by 1 to 2%; the rule's own margins are 2 to 8%.
+"""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_2603_25282_gb300 import inputs, sgp
+
+pytestmark = pytest.mark.gpu
+
+PRM = dict(omega=0.6, gamma=1.0, c0=400.0, c1=-1.0, c2=2.0)
+
+
+def _fastest(c, stream, runs):
+    """The least time of each run() over interleaved repetitions, in ms."""
+    best = [float("inf")] * len(runs)
+    for _ in range(6):
+        for k, run in enumerate(runs):
+            run()
+            c.synchronize()
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            with torch.cuda.stream(stream):
+                a.record()
+                run()
+                b.record()
+            b.synchronize()
+            best[k] = min(best[k], a.elapsed_time(b))
+    return best
+
+
+@pytest.mark.parametrize("n,batch", [((512, 128), 4), ((512, 128), 5), ((512, 128), 9), ((512, 128), 11),
+                                     ((1024, 128), 3), ((1024, 128), 5), ((512, 512), 1), ((512, 768), 1)])
+def test_long_rows(n, batch):
+    stream = torch.cuda.Stream()
+    psi = inputs.gaussian_random_phase(n, 8.0, seed=1).astype(np.complex64)
+    with sgp.Context(n, 8.0, batch=batch, stream=stream.cuda_stream) as c:
+        c.set_params(**PRM)
+        c.set_state(np.broadcast_to(psi, (batch,) + psi.shape).copy(), 0.0)
+
+        def steps(plan):
+            def run():
+                c.step(40, 1e-3, "ts2")
+            return plan, run
+
+        ms = {}
+        for plan, run in map(steps, [(0, 0), (1, 4), (7, 4)] * 2):
+            c.set_plan(plan)
+            ms[plan] = min(ms.get(plan, float("inf")), _fastest(c, stream, [run])[0])
+        assert ms[0, 0] <= 1.04 * min(ms[1, 4], ms[7, 4]), ms
