@@ -1218,12 +1218,12 @@ sgp_status record_steps(sgp_ctx* c, long long nsteps, double dt, int scheme, lon
 // Rows of the parameter partials per member: one per CTA of the adjoint
 // x-pass, then one per CTA of the line pass that holds the full transform
 // (y lines in 2D, z lines in 3D).
-// On grids whose passes are the FP32 component-parallel ones, a gradient's are
-// too, unless the plan has the plain kernels on some axis (variant 7).
+// On FP32 grids of the component-parallel passes' size a gradient's are too,
+// unless the plan has the plain kernels on some axis (variant 7).
 bool adj_split(const sgp_ctx* c) {
-  if (c->prec != SGP_F32) return false;
+  if (c->prec != SGP_F32 || !split_range(c->dim, c->ntot * c->batch)) return false;
   for (int a = 0; a < c->dim; ++a)
-    if (c->def[a] != kSplitPass || c->var[a] == 7) return false;
+    if (c->var[a] == 7) return false;
   return true;
 }
 template <typename R>
@@ -2212,7 +2212,8 @@ sgp_status sgp_create_grid(int dim, const int* n, const double* L, int batch, in
     else
       k_twiddles_f64<<<(c->n[a] + 255) / 256, 256, 0, c->stream>>>(c->n[a], E, (TwE<double>*)c->tw[a]);
     c->launches++;
-    if (c->def[a] < kSplitPass || (prec == SGP_F32 && split_elems_rt<float>(c->n[a]) == E)) continue;
+    // the radix plans of the component-parallel passes, a gradient's among them
+    if (prec == SGP_F32 && (!split_range(dim, c->ntot * batch) || split_elems_rt<float>(c->n[a]) == E)) continue;
     if ((e = dev_alloc(c, &c->tws[a], (size_t)c->n[a] * 16)) != cudaSuccess)
       return bail(SGP_ENOMEM, "twiddle allocation", e);
     if (prec == SGP_F32)

@@ -220,10 +220,16 @@ inline cudaError_t launch_linepass(int N, int V, const LPassArgs<R>& a, int plan
 // What variant 0 of an axis stands for, by the size of the whole batch (pts
 // grid points), the precision and the line length; measured per TS2 step on
 // the GB300 (plain variant 0 -> the choice, us):
-//   component-parallel passes for grids of few lines: FP32 2D up to 192 Ki
-//     points (64^2 22 -> 5, 256^2 32 -> 10, 384^2 44 -> 27; from 256 Ki points
-//     the others are ahead: 4 x 256^2 27 against 33), 3D below 128 Ki (48^3
-//     35 -> 28; 64 x 64 x 32 28 against 30);
+//   component-parallel passes for grids of few lines (split_range): FP32 2D up
+//     to 192 Ki points (64^2 22 -> 5, 256^2 32 -> 10, 384^2 44 -> 27; from 256
+//     Ki points the others are ahead: 4 x 256^2 27 against 33), 3D below 128 Ki
+//     (48^3 35 -> 28; 64 x 64 x 32 28 against 30).  Past 128 Ki points y-lines
+//     shorter than 64, whose CTAs of two columns are one to three warps, take
+//     geometry 2 unless the rows are the shortest (with component-parallel
+//     rows, split -> geometry 2: 32 x 48 times 128 30.7 -> 25.5, times 96 24.1 ->
+//     21.8, 64 x 32 times 72 19.0 -> 18.2, 96 x 16 times 128 27.0 -> 23.8, 1024 x
+//     32 times 5 27.1 -> 26.1, times 4 16.8 -> 17.6; but 16 x 16 times 768 26.9 ->
+//     37.5, and 64 x 64 times 40 20.0 -> 19.9);
 //   FP64 everywhere (fixed-point transforms, sgp_fix.cuh: 64^2 229 -> 50, 8 x
 //     512^2 5300 -> 2500, 128^3 5510 -> 2610), with one line per CTA while that
 //     gives no more than four CTAs an SM;
@@ -248,10 +254,16 @@ inline int long_row_geometry(int nx, long long rows, int sms) {
   return level && (nx <= 512 || c0 <= 2LL * sms) ? 0 : 1;
 }
 
+// FP32 grids (whole batches) of few lines
+inline bool split_range(int dim, long long pts) { return pts <= (dim == 2 ? 3LL << 16 : (1LL << 17) - 1); }
+
 inline int default_kernel(int prec_bytes, int dim, const int* n, int batch, int a, bool tensor_maps, int sms) {
   const long long pts = (long long)n[0] * n[1] * (dim == 3 ? n[2] : 1) * batch;
   if (prec_bytes == 8) return pts / n[a] > 4LL * sms ? kSplitMany : kSplitPass;
-  if (pts <= (dim == 2 ? 3LL << 16 : (1LL << 17) - 1)) return kSplitPass;
+  if (split_range(dim, pts)) {
+    const bool short_columns = dim == 2 && a == 1 && n[1] < 64 && n[0] >= 32;
+    return short_columns && pts > 8LL << 14 ? 2 : kSplitPass;
+  }
   if (dim == 3) return 1;
   if (a == 0) return n[0] >= 512 && n[0] % 3 != 0 ? long_row_geometry(n[0], pts / n[0], sms) : 1;
   return tensor_maps ? 4 : 1;
