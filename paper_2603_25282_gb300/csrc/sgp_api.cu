@@ -1218,13 +1218,14 @@ sgp_status record_steps(sgp_ctx* c, long long nsteps, double dt, int scheme, lon
 // Rows of the parameter partials per member: one per CTA of the adjoint
 // x-pass, then one per CTA of the line pass that holds the full transform
 // (y lines in 2D, z lines in 3D).
-// On FP32 grids of the component-parallel passes' size a gradient's are too,
-// unless the plan has the plain kernels on some axis (variant 7).
+// On FP32 grids of the component-parallel passes' size a gradient's are too
+// where they pay, unless the plan has the plain kernels on some axis (variant
+// 7).
 bool adj_split(const sgp_ctx* c) {
   if (c->prec != SGP_F32 || !split_range(c->dim, c->ntot * c->batch)) return false;
   for (int a = 0; a < c->dim; ++a)
     if (c->var[a] == 7) return false;
-  return true;
+  return gradient_split_pays(c->dim, c->n, c->batch, c->sms);
 }
 template <typename R>
 int adjoint_xrows(const sgp_ctx* c) {

@@ -269,6 +269,21 @@ inline int default_kernel(int prec_bytes, int dim, const int* n, int batch, int 
   return tensor_maps ? 4 : 1;
 }
 
+// Do a gradient's passes run component-parallel too?  In the range of split_range
+// (24 TS2 steps with the sweep, us, plain -> split: 64^2 1820 -> 550, 2 x 256^2
+// 2360 -> 1870, 48^3 3060 -> 2550) but for
+//   rows of 1024 points, whose adjoint CTAs (640 threads of 128 registers) are one
+//     to an SM: past one wave of rows (3 x 1024 x 48 2340 -> 2100, 4 x 1024 x 48
+//     2660 -> 3030);
+//   rows of 32 points, a CTA of one warp each: past 128 Ki points in 2D (32 x 64
+//     times 64 2000 -> 1940, times 96 2440 -> 2730), past 112 Ki in 3D (32 x 16 x
+//     16 times 15 2470 -> 2640).
+inline bool gradient_split_pays(int dim, const int* n, int batch, int sms) {
+  const long long pts = (long long)n[0] * n[1] * (dim == 3 ? n[2] : 1) * batch;
+  if (n[0] == 1024 && pts / n[0] > sms) return false;
+  return n[0] != 32 || pts <= (dim == 2 ? 8LL << 14 : 7LL << 14);
+}
+
 // Observables kernels (default geometry only).
 template <typename R>
 cudaError_t launch_obs_x(int N, const ObsXArgs<R>& a, int members, cudaStream_t s);
