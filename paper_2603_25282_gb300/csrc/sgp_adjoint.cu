@@ -149,24 +149,12 @@ k_linepass_adj(LPassArgs<R> a, AdjHook<R> h) {
   linepass_body<R, N, E, G, false, false, AdjHook<R>>(a, blockIdx.x, blockIdx.y, blockIdx.z, smem_raw, nullptr, h);
 }
 
-// Opt in to more than 48 KB of dynamic shared memory once per device.
-template <typename K>
-cudaError_t opt_in(K kern, size_t smem, int* done_dev) {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (*done_dev == dev) return cudaSuccess;
-  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e == cudaSuccess) *done_dev = dev;
-  return e;
-}
-
 template <int N>
 cudaError_t xadj_n(const XAdjArgs<Real>& a, int members, cudaStream_t s) {
   constexpr int E = elems_per_thread<Real, N>();
   typedef XCfg<Real, N, E, kXAdjGeom> Cfg;
-  static int done = -1;
-  const cudaError_t e = opt_in(k_xadj<Real, N, E>, Cfg::SMEM, &done);
+  static std::atomic<int> done{-1};
+  const cudaError_t e = opt_in(k_xadj<Real, N, E>, Cfg::SMEM, done);
   if (e != cudaSuccess) return e;
   dim3 grid((a.rows + Cfg::ROWS - 1) / Cfg::ROWS, members);
   k_xadj<Real, N, E><<<grid, kXAdjThreads, Cfg::SMEM, s>>>(a);
@@ -177,8 +165,8 @@ template <int N>
 cudaError_t xpass_tap_n(const XPassArgs<Real>& a, int members, cudaStream_t s) {
   constexpr int E = elems_per_thread<Real, N>();
   typedef XCfg<Real, N, E, kTapGeom> Cfg;
-  static int done = -1;
-  const cudaError_t e = opt_in(k_xpass_tap<Real, N, E>, Cfg::SMEM, &done);
+  static std::atomic<int> done{-1};
+  const cudaError_t e = opt_in(k_xpass_tap<Real, N, E>, Cfg::SMEM, done);
   if (e != cudaSuccess) return e;
   dim3 grid((a.rows + Cfg::ROWS - 1) / Cfg::ROWS, members);
   k_xpass_tap<Real, N, E><<<grid, Cfg::THREADS, Cfg::SMEM, s>>>(a);
@@ -194,8 +182,8 @@ cudaError_t linepass_adj_n(const LPassArgs<Real>& a, const AdjHook<Real>& h, int
   // the hook's staging sits behind the largest mode-table region
   constexpr size_t HB = AdjHook<Real>::smem_bytes<Real, N, Cfg::TILE>();
   static_assert(Cfg::SMEM + Cfg::TAB + HB <= 227 * 1024, "line pass of a gradient: shared memory");
-  static int done = -1;
-  const cudaError_t e = opt_in(k_linepass_adj<Real, N, E, G>, Cfg::SMEM + Cfg::TAB + HB, &done);
+  static std::atomic<int> done{-1};
+  const cudaError_t e = opt_in(k_linepass_adj<Real, N, E, G>, Cfg::SMEM + Cfg::TAB + HB, done);
   if (e != cudaSuccess) return e;
   dim3 grid((a.nx + Cfg::TILE - 1) / Cfg::TILE, planes, members);
   const size_t smem = Cfg::SMEM + Cfg::TAB + (h.spec ? HB : 0);

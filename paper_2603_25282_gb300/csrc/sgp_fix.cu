@@ -103,26 +103,15 @@ __global__ void k_fix_twiddles(int N, int E, FixTw* out) {
   out[k] = w;
 }
 
-template <typename K>
-cudaError_t opt_in(K kern, size_t smem, int* done_dev) {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (*done_dev == dev) return cudaSuccess;
-  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e == cudaSuccess) *done_dev = dev;
-  return e;
-}
-
 template <int N, int G>
 cudaError_t xfix_prepare() {
-  static int done = -1;
-  return opt_in(k_xfix<N, G>, FixCfg<N, G>::SMEM, &done);
+  static std::atomic<int> done{-1};
+  return opt_in(k_xfix<N, G>, FixCfg<N, G>::SMEM, done);
 }
 template <int N, int G>
 cudaError_t lfix_prepare() {
-  static int done = -1;
-  return opt_in(k_lfix<N, G>, FixCfg<N, G>::SMEM, &done);
+  static std::atomic<int> done{-1};
+  return opt_in(k_lfix<N, G>, FixCfg<N, G>::SMEM, done);
 }
 
 template <int N, int G>

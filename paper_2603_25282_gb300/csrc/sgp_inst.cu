@@ -19,20 +19,6 @@
 
 namespace sgp {
 
-namespace {
-// Opt in to more than 48 KB of dynamic shared memory once per device.
-template <typename K>
-cudaError_t prepare(K kern, size_t smem, int* done_dev) {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (*done_dev == dev) return cudaSuccess;
-  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e == cudaSuccess) *done_dev = dev;
-  return e;
-}
-}  // namespace
-
 typedef SGP_REAL Real;
 constexpr int V = SGP_VAR;
 
@@ -57,12 +43,12 @@ template <int N>
 static cudaError_t xpass_prepare_n() {
   constexpr int E = variant_elems<Real, N, V>();
   constexpr int G = variant_geom<N, V, SGP_PART>();
-  static int done = -1;
-  cudaError_t e = prepare(k_xpass<Real, N, E, G>, XCfg<Real, N, E, G>::SMEM, &done);
+  static std::atomic<int> done{-1};
+  cudaError_t e = opt_in(k_xpass<Real, N, E, G>, XCfg<Real, N, E, G>::SMEM, done);
 #if SGP_VAR == 0
   if (e != cudaSuccess) return e;
-  static int done_o = -1;
-  e = prepare(k_obs_x<Real, N, E>, XCfg<Real, N, E>::SMEM, &done_o);
+  static std::atomic<int> done_o{-1};
+  e = opt_in(k_obs_x<Real, N, E>, XCfg<Real, N, E>::SMEM, done_o);
 #endif
   return e;
 }
@@ -112,8 +98,8 @@ static_assert(sizeof(Real) == 4, "the xy-plane pass is FP32 only");
 template <int N>
 static cudaError_t xyplane_prepare_n() {
   typedef PlCfg<Real, N, elems_per_thread<Real, N>()> Cfg;
-  static int done = -1;
-  return prepare(k_xyplane<Real, N, elems_per_thread<Real, N>()>, Cfg::SMEM, &done);
+  static std::atomic<int> done{-1};
+  return opt_in(k_xyplane<Real, N, elems_per_thread<Real, N>()>, Cfg::SMEM, done);
 }
 
 template <int N>
@@ -151,8 +137,8 @@ cudaError_t launch_xyplane(int N, const XPassArgs<Real>& a, const TwE<Real>* twy
 template <int N>
 static cudaError_t xpass_wide_prepare_n() {
   constexpr int E = elems_per_thread<Real, N>();
-  static int done = -1;
-  return prepare(k_xpass_wide<Real, N, E>, XCfg<Real, N, E, 2>::SMEM, &done);
+  static std::atomic<int> done{-1};
+  return opt_in(k_xpass_wide<Real, N, E>, XCfg<Real, N, E, 2>::SMEM, done);
 }
 
 template <>
@@ -239,13 +225,12 @@ template <int N>
 static cudaError_t linepass_prepare_n() {
   constexpr int E = variant_elems<Real, N, V>();
   constexpr int G = variant_geom<N, V, SGP_PART>();
-  static int done = -1;
-  cudaError_t e = prepare(k_linepass<Real, N, E, G>,
-                          LCfg<Real, N, E, G>::SMEM + LCfg<Real, N, E, G>::TAB, &done);
+  static std::atomic<int> done{-1};
+  cudaError_t e = opt_in(k_linepass<Real, N, E, G>, LCfg<Real, N, E, G>::SMEM + LCfg<Real, N, E, G>::TAB, done);
 #if SGP_VAR == 0
   if (e != cudaSuccess) return e;
-  static int done_o = -1;
-  e = prepare(k_obs_line<Real, N, E>, LCfg<Real, N, E>::SMEM, &done_o);
+  static std::atomic<int> done_o{-1};
+  e = opt_in(k_obs_line<Real, N, E>, LCfg<Real, N, E>::SMEM, done_o);
 #endif
   return e;
 }
@@ -299,8 +284,8 @@ static_assert(sizeof(Real) == 4, "tensor-copy tile loads are FP32 only");
 template <int N>
 static cudaError_t linepass_tma_prepare_n() {
   constexpr int E = elems_per_thread<Real, N>();
-  static int done = -1;
-  return prepare(k_linepass_tma<Real, N, E, 1>, LCfg<Real, N, E, 1>::TSMEM + LCfg<Real, N, E, 1>::TAB, &done);
+  static std::atomic<int> done{-1};
+  return opt_in(k_linepass_tma<Real, N, E, 1>, LCfg<Real, N, E, 1>::TSMEM + LCfg<Real, N, E, 1>::TAB, done);
 }
 
 template <int N>

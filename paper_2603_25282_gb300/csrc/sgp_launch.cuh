@@ -4,6 +4,8 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <atomic>
+
 #include "sgp_kernels.cuh"
 
 namespace sgp {
@@ -85,6 +87,18 @@ struct PassGeom {
   int rows_or_tile;   // rows per CTA (x-pass) or columns per CTA (line pass)
   size_t smem;
 };
+
+// Lets a kernel have more than 48 KB of dynamic shared memory on the current
+// device; done: the device it was last done on (any number of host threads).
+template <typename K>
+inline cudaError_t opt_in(K kern, size_t smem, std::atomic<int>& done) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess || done.load(std::memory_order_acquire) == dev) return e;
+  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e == cudaSuccess) done.store(dev, std::memory_order_release);
+  return e;
+}
 
 // Launch of a pass kernel; dependent: it may begin while the pass before it on
 // the stream is at work (the kernel waits in pdl_wait before it touches the

@@ -7,22 +7,11 @@
 namespace sgp {
 namespace {
 
-template <typename K>
-cudaError_t opt_in(K kern, size_t smem, int* done_dev) {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (*done_dev == dev) return cudaSuccess;
-  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e == cudaSuccess) *done_dev = dev;
-  return e;
-}
-
 template <int N>
 cudaError_t xsplit_prepare_n() {
   constexpr int E = split_elems<float, N>(), G = split_rows<float, N>();
-  static int done = -1;
-  return opt_in(k_xsplit<float, N, E, G, false>, SplitCfg<float, N, E, G>::SMEM, &done);
+  static std::atomic<int> done{-1};
+  return opt_in(k_xsplit<float, N, E, G, false>, SplitCfg<float, N, E, G>::SMEM, done);
 }
 
 template <int N>
@@ -38,8 +27,8 @@ cudaError_t xsplit_n(const XPassArgs<float>& a, int members, bool dependent, cud
 template <int N>
 cudaError_t lsplit_prepare_n() {
   constexpr int E = split_elems<float, N>(), G = split_cols<float, N>();
-  static int done = -1;
-  return opt_in(k_lsplit<float, N, E, G, false, NoAdj>, SplitCfg<float, N, E, G>::SMEM, &done);
+  static std::atomic<int> done{-1};
+  return opt_in(k_lsplit<float, N, E, G, false, NoAdj>, SplitCfg<float, N, E, G>::SMEM, done);
 }
 
 template <int N>
@@ -56,16 +45,16 @@ cudaError_t lsplit_n(const LPassArgs<float>& a, int planes, int members, bool de
 template <int N>
 cudaError_t xadj_prepare_n() {
   constexpr int E = split_elems<float, N>(), G = split_rows<float, N>();
-  static int done = -1, done_t = -1;
-  const cudaError_t e = opt_in(k_xadj_split<float, N, E, G>, SplitCfg<float, N, E, G>::SMEM, &done);
+  static std::atomic<int> done{-1}, done_t{-1};
+  const cudaError_t e = opt_in(k_xadj_split<float, N, E, G>, SplitCfg<float, N, E, G>::SMEM, done);
   if (e != cudaSuccess) return e;
-  return opt_in(k_xsplit<float, N, E, G, true>, SplitCfg<float, N, E, G>::SMEM, &done_t);
+  return opt_in(k_xsplit<float, N, E, G, true>, SplitCfg<float, N, E, G>::SMEM, done_t);
 }
 template <int N>
 cudaError_t ladj_prepare_n() {
   constexpr int E = split_elems<float, N>(), G = split_cols<float, N>();
-  static int done = -1;
-  return opt_in(k_lsplit<float, N, E, G, true, AdjHook<float>>, SplitCfg<float, N, E, G>::SMEM, &done);
+  static std::atomic<int> done{-1};
+  return opt_in(k_lsplit<float, N, E, G, true, AdjHook<float>>, SplitCfg<float, N, E, G>::SMEM, done);
 }
 template <int N>
 cudaError_t xtap_n(const XPassArgs<float>& a, int members, bool dependent, cudaStream_t s) {
