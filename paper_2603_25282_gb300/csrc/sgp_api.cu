@@ -805,25 +805,29 @@ sgp_status line_pass_on(sgp_ctx* c, void* field, int axis, int mode, const LinTa
     static_cast<std::vector<PersistPass<R>>*>(c->rec)->push_back(p);
     return SGP_OK;
   }
+  int kern = axis_kernel(c, axis);
   if constexpr (sizeof(R) == 4) {
-    if (axis_kernel(c, axis) == 4) {
+    if (kern == 4) {
       // the batch the window's field belongs to (member coordinates mc0 + m)
       char* batch_base = (char*)field - (size_t)c->win0 * 5 * c->ntot * c->elem;
-      SGP_TRY(ensure_tmap(c, axis, batch_base));
-      c->launches++;
-      c->tiles = true;
-      ProfScope ps(c, axis == 1 ? PK_Y : PK_Z);
-      const bool dep = c->chain && !c->profiling;
-      c->chain = true;
-      SGP_CUDA(c, launch_linepass_tma(c->n[axis], a, c->tmap[axis], planes, window_members(c), dep, c->stream));
-      return SGP_OK;
+      const sgp_status st = ensure_tmap(c, axis, batch_base);
+      if (st == SGP_OK) {
+        c->launches++;
+        c->tiles = true;
+        ProfScope ps(c, axis == 1 ? PK_Y : PK_Z);
+        const bool dep = c->chain && !c->profiling;
+        c->chain = true;
+        SGP_CUDA(c, launch_linepass_tma(c->n[axis], a, c->tmap[axis], planes, window_members(c), dep, c->stream));
+        return SGP_OK;
+      }
+      if (c->var[axis] == 4) return st;
+      kern = 1;                         // variant 0 without a map: the same pass with plain loads
     }
   }
   c->launches++;
   ProfScope ps(c, axis == 1 ? PK_Y : PK_Z);
   const bool dep = c->chain && !c->profiling;
   c->chain = true;
-  const int kern = axis_kernel(c, axis);
   if (kern >= kSplitPass) {
     if (c->tws[axis]) a.tw = (const TwE<R>*)c->tws[axis];
     SGP_CUDA(c, launch_lsplit<R>(c->n[axis], kern != kSplitPass, a, planes, window_members(c), dep, c->stream));
