@@ -916,7 +916,8 @@ std::vector<SubRec> merged_substeps(int scheme, long long n, double dt) {
 }
 
 // Issue nsteps of the composition from the device time *t_dev and advance
-// it by nsteps*dt (or, with own_time, from run_t0), physical space in and out.  The merged substeps become
+// it by nsteps*dt (or, with own_time, from run_t0, which the caller advances),
+// physical space in and out.  The merged substeps become
 // passes: a nonlinear flow is an x-pass (inverse x-FFT if the field is
 // x-spectral, the flow, forward x-FFT if a linear flow follows); a linear
 // flow is the line passes on the x-spectral field (a forward x-pass first if
@@ -1073,18 +1074,17 @@ sgp_status substep(sgp_ctx* c, int kind, double delta) {
 // ----------------------------------------------------------------------------
 // The batch is split into `chunks` member groups.  All copies to the device
 // are issued on cs_in; each group's steps run after its copy has landed
-// (the passes restricted to the group by the member window), alternately
-// on the context stream and on cs_alt with its own device time, so that
-// the last passes of one group overlap the first of the next; each group's
-// copy back runs on cs_out after its steps.  The copy engines move group
-// k+1 in and group k-1 out while group k is propagated.
+// (the passes restricted to the group by the member window and carrying the
+// time in their arguments), alternately on the context stream and on cs_alt,
+// so that the last passes of one group overlap the first of the next; each
+// group's copy back runs on cs_out after its steps.  The copy engines move
+// group k+1 in and group k-1 out while group k is propagated.
 template <typename R>
 sgp_status step_host_impl(sgp_ctx* c, const void* hin, double t0, void* hout, long long nsteps,
                           double dt, int scheme, int chunks) {
   if (!c->cs_in) SGP_CUDA(c, cudaStreamCreateWithFlags(&c->cs_in, cudaStreamNonBlocking));
   if (!c->cs_out) SGP_CUDA(c, cudaStreamCreateWithFlags(&c->cs_out, cudaStreamNonBlocking));
   if (!c->cs_alt) SGP_CUDA(c, cudaStreamCreateWithFlags(&c->cs_alt, cudaStreamNonBlocking));
-  if (!c->t_dev_alt) SGP_CUDA(c, dev_alloc(c, (void**)&c->t_dev_alt, sizeof(double)));
   // the linear-flow tables of the run exist before the streams fork
   if (nsteps > 0) SGP_TRY(ensure_tables<R>(c, dt, scheme));
   const size_t nev = 2 * (size_t)chunks + 2;
@@ -1114,12 +1114,9 @@ sgp_status step_host_impl(sgp_ctx* c, const void* hin, double t0, void* hout, lo
   sgp_status st = SGP_OK;
   for (int k = 0; k < chunks && st == SGP_OK; ++k) {
     const size_t off = (size_t)m0[k] * mb, bytes = (size_t)(m0[k + 1] - m0[k]) * mb;
-    // odd groups on the second compute stream with its own device time
+    // odd groups on the second compute stream
     const bool alt = (k & 1) != 0;
-    if (alt) {
-      std::swap(c->stream, c->cs_alt);
-      std::swap(c->t_dev, c->t_dev_alt);
-    }
+    if (alt) std::swap(c->stream, c->cs_alt);
     cudaError_t e = cudaStreamWaitEvent(c->stream, ev[2 + k], 0);
     c->win0 = m0[k];
     c->wcnt = m0[k + 1] - m0[k];
@@ -1131,10 +1128,7 @@ sgp_status step_host_impl(sgp_ctx* c, const void* hin, double t0, void* hout, lo
     c->win0 = 0;
     c->wcnt = 0;
     if (st == SGP_OK) e = cudaEventRecord(ev[2 + chunks + k], c->stream);
-    if (alt) {
-      std::swap(c->stream, c->cs_alt);
-      std::swap(c->t_dev, c->t_dev_alt);
-    }
+    if (alt) std::swap(c->stream, c->cs_alt);
     if (st != SGP_OK) break;
     if (e == cudaSuccess) e = cudaStreamWaitEvent(c->cs_out, ev[2 + chunks + k], 0);
     if (e == cudaSuccess)
@@ -1217,9 +1211,6 @@ sgp_status record_steps(sgp_ctx* c, long long nsteps, double dt, int scheme, lon
   return SGP_OK;
 }
 
-// Rows of the parameter partials per member: one per CTA of the adjoint
-// x-pass, then one per CTA of the line pass that holds the full transform
-// (y lines in 2D, z lines in 3D).
 // On FP32 grids of the component-parallel passes' size a gradient's are too
 // where they pay, unless the plan has the plain kernels on some axis (variant
 // 7).
@@ -1229,6 +1220,9 @@ bool adj_split(const sgp_ctx* c) {
     if (c->var[a] == 7) return false;
   return gradient_split_pays(c->dim, c->n, c->batch, c->sms);
 }
+// Rows of the parameter partials per member: one per CTA of the adjoint
+// x-pass, then one per CTA of the line pass that holds the full transform
+// (y lines in 2D, z lines in 3D).
 template <typename R>
 int adjoint_xrows(const sgp_ctx* c) {
   const int rows = c->n[1] * c->n[2];

@@ -7,12 +7,16 @@
 // one common exponent, transformed in 64-bit integer arithmetic (an addition
 // is two instructions, a complex twiddle product twelve 32 x 32 -> 64 bit
 // multiply-adds), and brought back to doubles.  The common exponent follows
-// the line from stage to stage, so that its largest value has 57 bits or more
-// before every butterfly: rounding is below 2^-57 of the line's largest value,
-// against 2^-53 of each value in FP64, and a transform comes out closer to the
-// exact one than the FP64 transform does.  The pointwise flow and the
-// mode mix stay in FP64, with fewer operations than the forms that FP32 shares
-// (flow_point, mix_mode).
+// the line from stage to stage, so that its largest value has a modulus of 2^56
+// or more before every butterfly.  A line enters with 58 bits for its largest
+// component and 58 - k for one 2^-k of it, truncated; a twiddle product errs by
+// up to 1.5 units, one by sqrt(1/2) or sqrt(3)/2 by up to 2.5, and the floors add
+// up: an element of a random line of 768 comes out off by up to 2^-52.4 of the
+// line's largest value.  In relative L2 a transform is closer to the exact one
+// than in FP64 (an emulation of the integers: 2e-17 to 6e-17 for random lines, up
+// to 1.3e-16 for smooth ones of 768 and 1024; FP64 1.4e-16 to 2.4e-16).  The
+// pointwise flow and the mode mix stay in FP64, with fewer operations than the
+// forms that FP32 shares (flow_point, mix_mode).
 //
 // Measured (GB300; relative L2 of a forward and inverse 2D transform, and us
 // per launch): 256^2 3.3e-16 in FP64, 1.0e-16 here; 192 x 128 4.0e-16, 1.4e-16.
@@ -91,9 +95,10 @@ __device__ __forceinline__ longlong2 fix_twiddle(longlong2 x, FixTw w) {
 // ----------------------------------------------------------------------------
 // doubles to integers of a common exponent and back
 // ----------------------------------------------------------------------------
-// A line starts below 2^kFixStart and is brought to 2^kFixTw before each
-// twiddle stage, so below 2^58 before every butterfly: radix 8 stays below
-// 8 sqrt2 2^58 < 2^62, which the twiddle product of the next stage accepts.
+// A line's components start below 2^kFixStart and are brought below 2^kFixTw
+// (the largest to half of that or more) before each twiddle stage, so below
+// 2^57.5 before its butterflies: radix 8 stays below 8 sqrt2 2^58 < 2^62, which
+// the twiddle product of the next stage accepts.
 constexpr int kFixStart = 58, kFixTw = 59;
 constexpr int kFixBad = 1 << 20;        // exponent of a line that is not finite
 
@@ -467,9 +472,9 @@ __device__ __forceinline__ void mix_mode(double2 (&v)[5], const ModeEntry<double
 template <int N>
 constexpr int fix_elems() { return N % 3 == 0 ? 12 : N >= 512 ? 16 : 8; }
 
-// G lines of each component per CTA: one (two where a line is too short), for
-// grids of few lines; as many as make a warp per component otherwise (a CTA of
-// fewer threads spends more of its time on its constants and barriers).
+// G lines of each component per CTA: one for grids of few lines; as many as make
+// a warp per component otherwise (a CTA of fewer threads spends more of its time
+// on its constants and barriers).
 template <int N>
 constexpr int fix_lines(bool many) { return many && N / fix_elems<N>() < 32 ? 32 / (N / fix_elems<N>()) : 1; }
 

@@ -22,7 +22,8 @@
 namespace sgp {
 
 // Launches of at most this many CTAs let the next pass onto the SMs at once:
-// both then have SMs of their own (152 in all).  Larger ones wait until their
+// both then have SMs of their own (half the 152 of a GB300; a hint, on a device
+// with other numbers only the overlap differs).  Larger ones wait until their
 // points or modes are done, or the next pass crowds onto a few SMs (TS2 step,
 // one FP32 member: at 64^2 4.3 us early, 5.4 us late; at 256^2 12.0 and 10.4).
 constexpr unsigned kSplitEarly = 76;
@@ -424,8 +425,8 @@ constexpr int split_rows() { return N % 32 == 0 ? 1 : 2; }
 template <typename R, int N>
 constexpr int split_cols() { return N <= 512 ? 2 : 1; }
 // Elements per thread: those of the other passes, except 12 for N = 3*2^k:
-// radix 6 then 4s (192 = 6*4*4*2) instead of 6 then 2s (192 = 6*2*2*2*2*2), so
-// two stages fewer or more; one component's 12 elements are few registers.
+// radix 6 then 4s (192 = 6*4*4*2) instead of 6 then 2s (192 = 6*2*2*2*2*2), one
+// stage fewer for every factor 4; one component's 12 elements are few registers.
 template <typename R, int N>
 constexpr int split_elems() { return N % 3 == 0 ? 12 : 8; }
 // Launchers: FP32 here (sgp_split.cu); in FP64 the component-parallel passes
