@@ -3232,6 +3232,7 @@ sgp_status sgp_ensemble_observables(sgp_ens* e, sgp_obs* out) {
     sgp_ctx* c = e->groups[g];
     std::vector<sgp_obs> tmp(c->batch);
     sgp_status st = sgp_observables(c, tmp.data());
+    if (st == SGP_ETIMEOUT) e->have_state = false;
     if (st != SGP_OK && st != SGP_ENONFINITE) return efail(e, st, "%s", c->err.c_str());
     for (int m = 0; m < e->count; ++m)
       if (e->member_group[m] == (int)g) {

@@ -76,7 +76,7 @@ def test_default_kernels_report_it(words, call):
 def test_ensemble_reports_it(words):
     n = (128, 64)
     f = inputs.gaussian_random_phase(n, 8.0, seed=1).astype(np.complex64)
-    for call in ("get", "host", "sync"):
+    for call in ("get", "host", "sync", "observables"):
         with sgp.Ensemble([(n, 8.0)] * 2) as e:
             e.set_params([PRM] * 2)
             e.set_persistent(False)
@@ -90,8 +90,12 @@ def test_ensemble_reports_it(words):
                     e.get_member_state(0)
                 elif call == "host":
                     e.step_host([f, f], 0.0, 1, 1e-3)
+                elif call == "observables":
+                    e.observables()
                 else:
                     e.synchronize()
+            with pytest.raises(sgp.SgpError):
+                e.step(1, 1e-3)             # the states are undefined
             for m in (0, 1):
                 e.set_member_state(m, f, 0.0)
             e.step(1, 1e-3)
