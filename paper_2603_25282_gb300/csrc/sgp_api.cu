@@ -353,9 +353,11 @@ struct sgp_ctx {
   // first use) and the word a tile-load wait that gave up sets
   alignas(64) CUtensorMap tmap[3];
   const void* tmap_field[3] = {nullptr, nullptr, nullptr};   // the field a map was made for
-  // set by a tile-load wait that gave up; tiles: such loads have been issued or
-  // captured, so a result handed to the host is preceded by a look at err_dev
+  // set by a tile-load wait that gave up (it lies behind the sums of obs_dev, so
+  // that one copy brings both); tiles: such loads have been issued or captured,
+  // so a result handed to the host is preceded by a look at err_dev
   int* err_dev = nullptr;
+  int* err_host = nullptr;          // page-locked, for sgp_step_host
   bool tiles = false;
   int var[3] = {0, 0, 0};                        // kernel variant per axis (x-pass, y, z lines)
   // the kernel that variant 0 stands for on each axis (default_kernels), and
@@ -585,18 +587,22 @@ sgp_status get_tables(sgp_ctx* c, double delta, const LinTables** out) {
   return SGP_OK;
 }
 
-// Has a tile-load wait given up since the last look?  For calls that hand a
-// result to the host; the context's streams have been synchronised.
-sgp_status tile_status(sgp_ctx* c) {
-  if (!c->tiles) return SGP_OK;
-  int err = 0;
-  SGP_CUDA(c, cudaMemcpyAsync(&err, c->err_dev, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-  SGP_CUDA(c, cudaStreamSynchronize(c->stream));
+// Has a tile-load wait given up since the last look?  err: the error word, read
+// after the context's streams have been synchronised.
+sgp_status tile_report(sgp_ctx* c, int err) {
   if (!err) return SGP_OK;
   SGP_CUDA(c, cudaMemsetAsync(c->err_dev, 0, sizeof(int), c->stream));
   c->have_state = false;
   c->adj.valid = false;
   return fail(c, SGP_ETIMEOUT, "a tile-load wait of a pass gave up; the state is undefined until it is set again");
+}
+// The same for calls that hand a result to the host and read nothing else.
+sgp_status tile_status(sgp_ctx* c) {
+  if (!c->tiles) return SGP_OK;
+  int err = 0;
+  SGP_CUDA(c, cudaMemcpyAsync(&err, c->err_dev, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+  SGP_CUDA(c, cudaStreamSynchronize(c->stream));
+  return tile_report(c, err);
 }
 
 // ----------------------------------------------------------------------------
@@ -1085,6 +1091,7 @@ sgp_status step_host_impl(sgp_ctx* c, const void* hin, double t0, void* hout, lo
   if (!c->cs_in) SGP_CUDA(c, cudaStreamCreateWithFlags(&c->cs_in, cudaStreamNonBlocking));
   if (!c->cs_out) SGP_CUDA(c, cudaStreamCreateWithFlags(&c->cs_out, cudaStreamNonBlocking));
   if (!c->cs_alt) SGP_CUDA(c, cudaStreamCreateWithFlags(&c->cs_alt, cudaStreamNonBlocking));
+  if (!c->err_host) SGP_CUDA(c, cudaMallocHost((void**)&c->err_host, sizeof(int)));
   // the linear-flow tables of the run exist before the streams fork
   if (nsteps > 0) SGP_TRY(ensure_tables<R>(c, dt, scheme));
   const size_t nev = 2 * (size_t)chunks + 2;
@@ -1141,6 +1148,10 @@ sgp_status step_host_impl(sgp_ctx* c, const void* hin, double t0, void* hout, lo
   // buffers are done with when this returns, also after an error
   cudaError_t e = cudaEventRecord(ev[1], c->cs_out);
   if (e == cudaSuccess) e = cudaStreamWaitEvent(c->stream, ev[1], 0);
+  // the error word on its way with the last copies
+  *c->err_host = 0;
+  if (c->tiles && e == cudaSuccess)
+    e = cudaMemcpyAsync(c->err_host, c->err_dev, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
   const cudaError_t e1 = cudaStreamSynchronize(c->cs_in);
   const cudaError_t e2 = cudaStreamSynchronize(c->cs_out);
   const cudaError_t e3 = cudaStreamSynchronize(c->stream);
@@ -1148,7 +1159,7 @@ sgp_status step_host_impl(sgp_ctx* c, const void* hin, double t0, void* hout, lo
   if (st != SGP_OK) return st;
   for (cudaError_t x : {e, e1, e2, e3, e4})
     if (x != cudaSuccess) return fail(c, SGP_ECUDA, "sgp_step_host: %s", cudaGetErrorString(x));
-  return tile_status(c);
+  return tile_report(c, *c->err_host);
 }
 
 // ----------------------------------------------------------------------------
@@ -2064,11 +2075,13 @@ sgp_status observables(sgp_ctx* c, sgp_obs* out) {
         c->partials, al.nblocks, OBL_NT, c->obs_dev, OB_NT, axis == 1 ? OB_KY : OB_KZ);
     SGP_CUDA(c, cudaGetLastError());
   }
-  std::vector<double> h((size_t)c->batch * OB_NT, 0.0);
+  std::vector<double> h((size_t)c->batch * OB_NT + 1, 0.0);
   SGP_CUDA(c, cudaMemcpyAsync(h.data(), c->obs_dev, h.size() * sizeof(double),
                               cudaMemcpyDeviceToHost, c->stream));
   SGP_CUDA(c, cudaStreamSynchronize(c->stream));
-  SGP_TRY(tile_status(c));
+  int err = 0;
+  memcpy(&err, &h.back(), sizeof err);
+  SGP_TRY(tile_report(c, err));
   const double cell = c->h[0] * c->h[1] * (c->dim == 3 ? c->h[2] : 1.0);
   bool finite = true;
   for (int m = 0; m < c->batch; ++m) {
@@ -2222,10 +2235,6 @@ sgp_status sgp_create_grid(int dim, const int* n, const double* L, int batch, in
   }
   if ((e = dev_alloc(c, (void**)&c->t_dev, sizeof(double))) != cudaSuccess)
     return bail(SGP_ENOMEM, "time allocation", e);
-  if ((e = dev_alloc(c, (void**)&c->err_dev, sizeof(int))) != cudaSuccess)
-    return bail(SGP_ENOMEM, "error word allocation", e);
-  if ((e = cudaMemsetAsync(c->err_dev, 0, sizeof(int), c->stream)) != cudaSuccess)
-    return bail(SGP_ECUDA, "error word clear", e);
   if ((e = dev_alloc(c, (void**)&c->mp_dev, sizeof(MemberPrm) * batch)) != cudaSuccess)
     return bail(SGP_ENOMEM, "parameter allocation", e);
   // observables scratch: the largest per-kernel partial array
@@ -2240,11 +2249,12 @@ sgp_status sgp_create_grid(int dim, const int* n, const double* L, int batch, in
   c->partials_len = need * batch;
   if ((e = dev_alloc(c, (void**)&c->partials, c->partials_len * sizeof(double))) != cudaSuccess)
     return bail(SGP_ENOMEM, "observables scratch", e);
-  if ((e = dev_alloc(c, (void**)&c->obs_dev, (size_t)batch * OB_NT * sizeof(double))) != cudaSuccess)
+  const size_t obs_bytes = ((size_t)batch * OB_NT + 1) * sizeof(double);
+  if ((e = dev_alloc(c, (void**)&c->obs_dev, obs_bytes)) != cudaSuccess)
     return bail(SGP_ENOMEM, "observables output", e);
-  if ((e = cudaMemsetAsync(c->obs_dev, 0, (size_t)batch * OB_NT * sizeof(double), c->stream)) !=
-      cudaSuccess)
+  if ((e = cudaMemsetAsync(c->obs_dev, 0, obs_bytes, c->stream)) != cudaSuccess)
     return bail(SGP_ECUDA, "observables clear", e);
+  c->err_dev = reinterpret_cast<int*>(c->obs_dev + (size_t)batch * OB_NT);
   if ((e = cudaGetLastError()) != cudaSuccess) return bail(SGP_ECUDA, "table launch", e);
   if ((e = cudaStreamSynchronize(c->stream)) != cudaSuccess) return bail(SGP_ECUDA, "create sync", e);
   if (upload_params(c) != SGP_OK) {
@@ -2536,10 +2546,10 @@ sgp_status sgp_destroy(sgp_ctx* c) {
   for (void* t : c->tw4) dev_free(c, t);
   for (void* t : c->tws) dev_free(c, t);
   dev_free(c, c->t_dev);
-  dev_free(c, c->err_dev);
   dev_free(c, c->mp_dev);
   dev_free(c, c->partials);
   dev_free(c, c->obs_dev);
+  if (c->err_host) cudaFreeHost(c->err_host);
   dev_free(c, c->mass_dev);
   recycle_events(c);
   for (cudaEvent_t e : c->event_pool) cudaEventDestroy(e);

@@ -14,9 +14,13 @@ pytestmark = pytest.mark.gpu
 PRM = dict(omega=0.5, gamma=1.0, c0=100.0, c1=-1.0, c2=2.0)
 
 
+# 19 sums per member, then the error word
+OBS_BLOCK = {(19 * batch + 1) * 8 for batch in (1, 2)}
+
+
 @pytest.fixture
 def words():
-    """The 4-byte blocks that contexts take: their error words."""
+    """The error words of contexts of one or two members."""
     held = {}
 
     def _alloc(size, device, stream, user):
@@ -26,11 +30,12 @@ def words():
 
     keep = (sgp.ALLOC_FN(_alloc), sgp.FREE_FN(lambda p, *a: held.pop(p, None)))
     assert sgp.lib().sgp_set_allocator(keep[0], keep[1], None) == 0
-    yield lambda: [t[:4].view(torch.int32) for size, t in held.values() if size == 4]
+    yield lambda: [t[size - 8:size - 4].view(torch.int32) for size, t in held.values() if size in OBS_BLOCK]
     sgp.use_torch_allocator(False)
 
 
 def _set(words):
+    assert len(words()) == 1
     for w in words():
         w.fill_(1)
     torch.cuda.synchronize()
