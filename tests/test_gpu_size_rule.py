@@ -17,58 +17,50 @@ pytestmark = pytest.mark.gpu
 PRM = dict(omega=0.6, gamma=1.0, c0=400.0, c1=-1.0, c2=2.0)
 
 
-def _fastest(c, stream, runs):
-    """The least time of each run() over interleaved repetitions, in ms."""
-    best = [float("inf")] * len(runs)
-    for _ in range(6):
-        for k, run in enumerate(runs):
-            run()
-            c.synchronize()
-            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
-            with torch.cuda.stream(stream):
-                a.record()
+def _not_behind(c, stream, run, plans, bound):
+    """Is run() under plans[0] within bound of the fastest of the others?  Least
+    times of interleaved repetitions; more of them while the answer is no, since
+    another's work on the host can only add time."""
+    ms = dict.fromkeys(plans, float("inf"))
+    for _ in range(5):
+        for plan in plans * 2:
+            c.set_plan(plan)
+            for _ in range(6):
                 run()
-                b.record()
-            b.synchronize()
-            best[k] = min(best[k], a.elapsed_time(b))
-    return best
+                c.synchronize()
+                a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+                with torch.cuda.stream(stream):
+                    a.record()
+                    run()
+                    b.record()
+                b.synchronize()
+                ms[plan] = min(ms[plan], a.elapsed_time(b))
+        if ms[plans[0]] <= bound * min(ms[p] for p in plans[1:]):
+            return True
+    print(ms)
+    return False
 
 
-@pytest.mark.parametrize("n,batch", [((512, 128), 4), ((512, 128), 5), ((512, 128), 9), ((512, 128), 11),
-                                     ((1024, 128), 3), ((1024, 128), 5), ((512, 512), 1), ((512, 768), 1)])
-def test_long_rows(n, batch):
+def _steps(n, batch, plans):
     stream = torch.cuda.Stream()
     psi = inputs.gaussian_random_phase(n, 8.0, seed=1).astype(np.complex64)
     with sgp.Context(n, 8.0, batch=batch, stream=stream.cuda_stream) as c:
         c.set_params(**PRM)
         c.set_state(np.broadcast_to(psi, (batch,) + psi.shape).copy(), 0.0)
+        return _not_behind(c, stream, lambda: c.step(40, 1e-3, "ts2"), plans, 1.04)
 
-        def steps(plan):
-            def run():
-                c.step(40, 1e-3, "ts2")
-            return plan, run
 
-        ms = {}
-        for plan, run in map(steps, [(0, 0), (1, 4), (7, 4)] * 2):
-            c.set_plan(plan)
-            ms[plan] = min(ms.get(plan, float("inf")), _fastest(c, stream, [run])[0])
-        assert ms[0, 0] <= 1.04 * min(ms[1, 4], ms[7, 4]), ms
+@pytest.mark.parametrize("n,batch", [((512, 128), 4), ((512, 128), 5), ((512, 128), 9), ((512, 128), 11),
+                                     ((1024, 128), 3), ((1024, 128), 5), ((512, 512), 1), ((512, 768), 1)])
+def test_long_rows(n, batch):
+    assert _steps(n, batch, [(0, 0), (1, 4), (7, 4)])
 
 
 @pytest.mark.parametrize("n,batch", [((32, 48), 96), ((32, 48), 128), ((96, 16), 128), ((1024, 48), 4), ((64, 32), 72),
                                      ((16, 16), 768), ((64, 32), 56)])
 def test_short_columns(n, batch):
     """y-lines shorter than 64 on both sides of the line at 128 Ki points."""
-    stream = torch.cuda.Stream()
-    psi = inputs.gaussian_random_phase(n, 8.0, seed=1).astype(np.complex64)
-    with sgp.Context(n, 8.0, batch=batch, stream=stream.cuda_stream) as c:
-        c.set_params(**PRM)
-        c.set_state(np.broadcast_to(psi, (batch,) + psi.shape).copy(), 0.0)
-        ms = {}
-        for plan in [(0, 0), (0, 2)] * 2:
-            c.set_plan(plan)
-            ms[plan] = min(ms.get(plan, float("inf")), _fastest(c, stream, [lambda: c.step(40, 1e-3, "ts2")])[0])
-        assert ms[0, 0] <= 1.04 * ms[0, 2], ms
+    assert _steps(n, batch, [(0, 0), (0, 2)])
 
 
 def test_short_columns_result():
@@ -110,8 +102,4 @@ def test_gradients(n, batch):
             c.record(24, 1e-3, "ts2")
             c.backward(f, out)
 
-        ms = {}
-        for plan in (0, 7) * 2:
-            c.set_plan((plan,) * len(n))
-            ms[plan] = min(ms.get(plan, float("inf")), _fastest(c, stream, [run])[0])
-        assert ms[0] <= 1.08 * ms[7], ms
+        assert _not_behind(c, stream, run, [(0,) * len(n), (7,) * len(n)], 1.08)
